@@ -25,7 +25,7 @@
 #include <mutex>
 
 #include "runtime.h"
-#include "tube.cuh"
+#include "walk.cuh"
 
 namespace et {
 
@@ -34,126 +34,213 @@ namespace {
 constexpr long long NA_MAX_GRAINS = ET_NOALLOC_MAX_GRAINS;
 constexpr long long NA_MAX_CELLS = ET_NOALLOC_MAX_CELLS;
 
+// Two cell lists (rows along x and along y, as the regular path's) of at most
+// half the cells each.
+constexpr long long NA_LIST_CELLS = NA_MAX_CELLS / 2;
+
 // Layout of the scratch array (byte offsets, 256-aligned).
-constexpr size_t NA_OFF_GRAINS = 0;                                              // int4[MAX_GRAINS]
-constexpr size_t NA_OFF_START = NA_OFF_GRAINS + sizeof(int4) * NA_MAX_GRAINS;    // u32[MAX_CELLS + 1]
-constexpr size_t NA_OFF_CURSOR = NA_OFF_START + ((sizeof(u32) * (NA_MAX_CELLS + 1) + 255) / 256) * 256;
-constexpr size_t NA_OFF_FLAG = NA_OFF_CURSOR + sizeof(u32) * NA_MAX_CELLS;       // u32 error word
-constexpr size_t NA_BYTES = NA_OFF_FLAG + 256;
+constexpr size_t NA_ALIGN = 256;
+constexpr size_t na_up(size_t v) { return (v + NA_ALIGN - 1) / NA_ALIGN * NA_ALIGN; }
+constexpr size_t NA_OFF_GRAINS = 0;                                                       // u64[2 MAX_GRAINS]
+constexpr size_t NA_OFF_START = NA_OFF_GRAINS + sizeof(u64) * 2 * NA_MAX_GRAINS;          // u32[2][LIST_CELLS + 1]
+constexpr size_t NA_START_BYTES = na_up(sizeof(u32) * (NA_LIST_CELLS + 1));
+constexpr size_t NA_OFF_CURSOR = NA_OFF_START + 2 * NA_START_BYTES;                       // u32[2][LIST_CELLS]
+constexpr size_t NA_OFF_CTL = NA_OFF_CURSOR + sizeof(u32) * NA_MAX_CELLS;                 // NaCtl
+constexpr size_t NA_BYTES = NA_OFF_CTL + NA_ALIGN;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NA_BYTES];
 
+struct NaCtl {
+    u64 ticket;   // pairs taken by the counting warps
+    u32 bad;      // a coordinate lies outside the extent
+};
+
 struct NaScratch {
-    int4 *grains;
-    u32 *start;
-    u32 *cursor;
-    u32 *flag;
+    u64 *grains;               // packed, x-row list then (at N) y-row list
+    u32 *start[2], *cursor[2];
+    NaCtl *ctl;
 };
 
 NaScratch carve(unsigned char *base) {
     NaScratch s;
-    s.grains = (int4 *)(base + NA_OFF_GRAINS);
-    s.start = (u32 *)(base + NA_OFF_START);
-    s.cursor = (u32 *)(base + NA_OFF_CURSOR);
-    s.flag = (u32 *)(base + NA_OFF_FLAG);
+    s.grains = (u64 *)(base + NA_OFF_GRAINS);
+    for (int l = 0; l < 2; ++l) {
+        s.start[l] = (u32 *)(base + NA_OFF_START + l * NA_START_BYTES);
+        s.cursor[l] = (u32 *)(base + NA_OFF_CURSOR) + l * NA_LIST_CELLS;
+    }
+    s.ctl = (NaCtl *)(base + NA_OFF_CTL);
     return s;
 }
 
-__global__ void k_na_clear(NaScratch s, int ncell) {
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c <= ncell; c += gridDim.x * blockDim.x) {
-        s.start[c] = 0;
-        if (c < ncell) s.cursor[c] = 0;
+__global__ void k_na_clear(NaScratch s, int n0, int n1) {
+    griddep_launch();
+    griddep_wait();
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < max(n0, n1); c += gridDim.x * blockDim.x) {
+        if (c < n0) s.cursor[0][c] = 0;
+        if (c < n1) s.cursor[1][c] = 0;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) *s.flag = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        s.ctl->ticket = 0;
+        s.ctl->bad = 0;
+    }
 }
 
-__device__ __forceinline__ int na_cell(const Batch &b, int x, int y, int z) {
-    const int cx = min(x / b.cs[0], b.nc[0] - 1), cy = min(y / b.cs[1], b.nc[1] - 1);
-    const int cz = min(z / b.cs[2], b.nc[2] - 1);
-    return cx + b.nc[0] * (cy + b.nc[1] * cz);
+__device__ __forceinline__ bool na_inside(const Batch &b, int x, int y, int z) {
+    return x >= 0 && x < b.ext[0] && y >= 0 && y < b.ext[1] && z >= 0 && z < b.ext[2];
+}
+__device__ __forceinline__ int na_cell_x(const Batch &b, int x, int y, int z) {
+    return x / b.cs[0] + b.nc[0] * (y / b.cs[1] + b.nc[1] * (z / b.cs[2]));
+}
+__device__ __forceinline__ int na_cell_y(const Batch &b, int x, int y, int z) {
+    return y / b.csy[1] + b.ncy[1] * (x / b.csy[0] + b.ncy[0] * (z / b.csy[2]));
 }
 
 __global__ void k_na_count(Batch b, const int *xyz, NaScratch s) {
+    griddep_launch();
+    griddep_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < b.N; i += gridDim.x * blockDim.x) {
         const int x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
-        if (x < 0 || x >= b.ext[0] || y < 0 || y >= b.ext[1] || z < 0 || z >= b.ext[2]) {
-            atomicOr(s.flag, 1u);
+        if (!na_inside(b, x, y, z)) {
+            atomicOr(&s.ctl->bad, 1u);
             continue;
         }
-        atomicAdd(&s.cursor[na_cell(b, x, y, z)], 1u);
+        atomicAdd(&s.cursor[0][na_cell_x(b, x, y, z)], 1u);
+        atomicAdd(&s.cursor[1][na_cell_y(b, x, y, z)], 1u);
     }
 }
 
-// One block: exclusive scan of the per-cell counts into cell starts; the
-// counts are turned into fill cursors at the same time.
-__global__ void k_na_scan(NaScratch s, int ncell) {
-    __shared__ u32 part[1024];
-    __shared__ u32 carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < ncell; base += 1024) {
-        const int c = base + threadIdx.x;
-        const u32 v = c < ncell ? s.cursor[c] : 0u;
-        part[threadIdx.x] = v;
-        __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {   // Hillis-Steele inclusive scan
-            const u32 add = threadIdx.x >= o ? part[threadIdx.x - o] : 0u;
-            __syncthreads();
-            part[threadIdx.x] += add;
-            __syncthreads();
+// Block l scans the cell counts of list l into cell starts, which also become
+// the fill cursors: tiles of NA_SC x 1024 cells, the next tile's counts loaded
+// before the current one is scanned.  28k grains on 2 x 76k cells take 7 us; a
+// one-thread-per-cell shared-memory scan of one list took 53 us.
+constexpr int NA_SC = 8;
+
+__global__ void __launch_bounds__(1024) k_na_scan(NaScratch s, int n0, int n1) {
+    griddep_launch();
+    griddep_wait();
+    __shared__ u32 part[32];
+    const int list = blockIdx.x, n = list ? n1 : n0, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    u32 *cur = s.cursor[list], *start = s.start[list];
+    u32 carry = 0, v[NA_SC], next[NA_SC];
+    auto load = [&](int base, u32 (&d)[NA_SC]) {
+        const int c = base + (int)threadIdx.x * NA_SC;
+#pragma unroll
+        for (int k = 0; k < NA_SC; ++k) d[k] = c + k < n ? cur[c + k] : 0u;
+    };
+    load(0, next);
+    for (int base = 0; base < n; base += 1024 * NA_SC) {
+        u32 sum = 0;
+#pragma unroll
+        for (int k = 0; k < NA_SC; ++k) {
+            v[k] = next[k];
+            sum += v[k];
         }
-        const u32 ex = carry + part[threadIdx.x] - v;
-        if (c < ncell) {
-            s.start[c] = ex;
-            s.cursor[c] = ex;
+        load(base + 1024 * NA_SC, next);
+        u32 inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const u32 t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
         }
+        if (lane == 31) part[w] = inc;
         __syncthreads();
-        if (threadIdx.x == 1023) carry += part[1023];
-        __syncthreads();
+        u32 ps = part[lane];   // every warp scans the warp sums itself
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const u32 t = __shfl_up_sync(0xffffffffu, ps, o);
+            if (lane >= o) ps += t;
+        }
+        const u32 before = w ? __shfl_sync(0xffffffffu, ps, w - 1) : 0u;
+        u32 run = carry + before + inc - sum;
+        carry += __shfl_sync(0xffffffffu, ps, 31);
+        const int c = base + (int)threadIdx.x * NA_SC;
+#pragma unroll
+        for (int k = 0; k < NA_SC; ++k) {
+            if (c + k < n) {
+                start[c + k] = run;
+                cur[c + k] = run;
+            }
+            run += v[k];
+        }
+        __syncthreads();   // part is written again
     }
-    if (threadIdx.x == 0) s.start[ncell] = carry;
+    if (threadIdx.x == 0) start[n] = carry;
 }
 
 __global__ void k_na_scatter(Batch b, const int *xyz, NaScratch s) {
+    griddep_launch();
+    griddep_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < b.N; i += gridDim.x * blockDim.x) {
         const int x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
-        if (x < 0 || x >= b.ext[0] || y < 0 || y >= b.ext[1] || z < 0 || z >= b.ext[2]) continue;
-        const u32 pos = atomicAdd(&s.cursor[na_cell(b, x, y, z)], 1u);
-        s.grains[pos] = make_int4(x, y, z, i);
+        if (!na_inside(b, x, y, z)) continue;
+        const u64 g = pack_xyz(x, y, z);
+        s.grains[atomicAdd(&s.cursor[0][na_cell_x(b, x, y, z)], 1u)] = g;
+        s.grains[(u32)b.N + atomicAdd(&s.cursor[1][na_cell_y(b, x, y, z)], 1u)] = g;
     }
 }
 
-// One thread per pair: the exact tube test over the conservative cell cover.
+// The tube walk of the regular path (walk.cuh) over the caller's pairs: a warp
+// takes 32 pairs (fewer, at least 4, when there are too few to give every warp
+// 32) and deals their cell rows and grains over its lanes.
 // A pair with an index outside [0, n) or equal indices, a pair whose two
 // grains coincide or lie seed_max or more apart on some axis, and every pair
 // when a coordinate was out of range, gets -1.  The separation bound keeps
 // every cross-product component an exact int32 (|d_e w_f| + |d_f w_e| <
 // (extent_e + extent_f) seed_max < 2^31, the parameter precondition) and the
 // squared norms within 64 bits, as for the seeds of the regular path.
-__global__ void k_na_tube(Batch b, const int *xyz, const int *pairs, long long n_pairs, int *counts,
-                          NaScratch s) {
-    const bool bad_view = *(volatile u32 *)s.flag != 0;
-    for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n_pairs;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int i = pairs[2 * k], j = pairs[2 * k + 1];
-        if (bad_view || i < 0 || i >= b.N || j < 0 || j >= b.N || i == j) {
-            counts[k] = -1;
-            continue;
+// Bound by instruction issue like the regular tube counts.  With one thread
+// per pair the lanes of a warp waited for the longest of 32 walks: 400,001
+// pairs of a 28k-grain view took 377 us of a 431 us call; the call now takes
+// 193 us.
+constexpr int NA_W = 8;   // warps per block
+
+__global__ void __launch_bounds__(NA_W * 32, 4) k_na_tube(Batch b, const int *xyz, const int *pairs,
+                                                          long long n_pairs, int *counts, NaScratch s) {
+    griddep_launch();
+    griddep_wait();
+    __shared__ SeedTab sp[NA_W];
+    __shared__ int4 tbl[NA_W][32];
+    __shared__ u32 scount[NA_W][32];
+    __shared__ int nit[NA_W][32];   // items of each line
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const bool bad_view = *(volatile u32 *)&s.ctl->bad != 0;
+    const long long nwarps = (long long)gridDim.x * NA_W;
+    const int lines = (int)max(4ll, min(32ll, (n_pairs + nwarps - 1) / nwarps));
+    for (;;) {
+        u64 k0 = 0;
+        if (lane == 0) k0 = atomicAdd(&s.ctl->ticket, (u64)lines);
+        k0 = __shfl_sync(0xffffffffu, k0, 0);
+        if (k0 >= (u64)n_pairs) break;
+        const u64 k = k0 + lane;
+        const bool mine = lane < lines && k < (u64)n_pairs;
+        bool good = false;
+        int4 a = make_int4(0, 0, 0, 0), c = a;
+        if (mine) {
+            const int i = pairs[2 * k], j = pairs[2 * k + 1];
+            if (!bad_view && i >= 0 && i < b.N && j >= 0 && j < b.N && i != j) {
+                a = make_int4(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], 0);
+                c = make_int4(xyz[3 * j], xyz[3 * j + 1], xyz[3 * j + 2], 0);
+                const int dx = abs(c.x - a.x), dy = abs(c.y - a.y), dz = abs(c.z - a.z);
+                good = (dx | dy | dz) != 0 && dx < b.smax && dy < b.smax && dz < b.smax;
+            }
         }
-        const int3 a = make_int3(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2]);
-        const int3 d = make_int3(xyz[3 * j] - a.x, xyz[3 * j + 1] - a.y, xyz[3 * j + 2] - a.z);
-        if ((d.x == 0 && d.y == 0 && d.z == 0) || abs(d.x) >= b.smax || abs(d.y) >= b.smax ||
-            abs(d.z) >= b.smax) {
-            counts[k] = -1;
-            continue;
+        // the walk's lines are the first lanes', so the pairs to count move up
+        // past the others
+        const unsigned gm = __ballot_sync(0xffffffffu, good);
+        const int slot = __popc(gm & ((1u << lane) - 1u));
+        scount[wib][lane] = 0;
+        if (good) {
+            SeedSm q;
+            nit[wib][slot] = seed_setup(b, a, c, 0, q);
+            sp[wib].put(slot, q);
         }
-        const long long R = b.r2 * ((long long)d.x * d.x + (long long)d.y * d.y + (long long)d.z * d.z);
-        int c = 0;
-        const int4 *__restrict__ g = s.grains;
-        tube_cover(b, s.start, a, d, [&](u32 beg, u32 end) {
-            for (u32 q = beg; q < end; ++q) c += in_tube(g[q], a, d, R);
-        });
-        counts[k] = c;
+        __syncwarp();
+        u32 tests = 0;
+        warp_items<true, true, WALK_SERIAL>(b, sp[wib], tbl[wib], lane < __popc(gm) ? nit[wib][lane] : 0, tests,
+                                            scount[wib], [&](int own, int4) { atomicAdd(&scount[wib][own], 1u); });
+        __syncwarp();
+        if (mine) counts[k] = good ? (int)scount[wib][slot] : -1;
+        __syncwarp();
     }
 }
 
@@ -216,7 +303,8 @@ extern "C" et_status et_tube_count_noalloc(const int32_t *d_xyz, int64_t n, cons
         }
         base = g_na_base[dev];
     }
-    // cell grid: about one grain per cell, coarsened until it fits the scratch limit
+    // cell grid: the regular path's automatic shape, coarsened until both lists
+    // fit the scratch limit
     Batch b;
     memset(&b, 0, sizeof b);
     b.V = 1;
@@ -226,32 +314,43 @@ extern "C" et_status et_tube_count_noalloc(const int32_t *d_xyz, int64_t n, cons
     b.r2 = (long long)params->tube_r * params->tube_r;
     b.smax = params->seed_max;
     const double vol = (double)b.ext[0] * b.ext[1] * b.ext[2];
-    double sz = std::cbrt(vol / (double)std::max<int64_t>(n, 1));
-    long long ncell = 0;
+    double s0 = std::cbrt(0.35 * vol / (double)std::max<int64_t>(n, 1));
+    long long nx = 0, ny = 0;
     for (int tries = 0; tries < 64; ++tries) {
-        ncell = 1;
+        static const double f[3] = {0.2, 1.7, 1.4};
+        nx = ny = 1;
+        for (int k = 0; k < 3; ++k) b.cs[k] = (int)std::min<double>(std::max(1.0, std::round(s0 * f[k])), b.ext[k]);
+        b.csy[0] = std::min(b.cs[1], b.ext[0]);
+        b.csy[1] = std::min(b.cs[0], b.ext[1]);
+        b.csy[2] = b.cs[2];
         for (int k = 0; k < 3; ++k) {
-            b.cs[k] = std::max(1, std::min((int)std::ceil(sz), b.ext[k]));
             b.nc[k] = (b.ext[k] + b.cs[k] - 1) / b.cs[k];
+            b.ncy[k] = (b.ext[k] + b.csy[k] - 1) / b.csy[k];
             b.ics[k] = 1.0f / (float)b.cs[k];
-            ncell *= b.nc[k];
+            b.icsy[k] = 1.0f / (float)b.csy[k];
+            nx *= b.nc[k];
+            ny *= b.ncy[k];
         }
-        if (ncell <= NA_MAX_CELLS) break;
-        sz *= 1.26;
+        if (std::max(nx, ny) <= NA_LIST_CELLS) break;
+        s0 *= 1.26;
     }
-    if (ncell > NA_MAX_CELLS) return fail(ET_ERR_INVALID_ARG, "no cell grid fits the fixed scratch limit");
-    b.ncell = (int)ncell;
+    if (std::max(nx, ny) > NA_LIST_CELLS) return fail(ET_ERR_INVALID_ARG, "no cell grid fits the fixed scratch limit");
+    b.ncell = (int)nx;
+    b.ncelly = (int)ny;
+    b.dual = 1;
     const NaScratch s = carve(base);
+    b.cell_start = s.start[0];
+    b.cell_start_y = s.start[1];
+    b.gp = s.grains;
     cudaStream_t cst = (cudaStream_t)stream;
-    k_na_clear<<<64, 256, 0, cst>>>(s, (int)ncell);
-    if (n > 0) {
-        const unsigned gn = (unsigned)std::min<long long>((n + 255) / 256, 1024);
-        k_na_count<<<gn, 256, 0, cst>>>(b, d_xyz, s);
-        k_na_scan<<<1, 1024, 0, cst>>>(s, (int)ncell);
-        k_na_scatter<<<gn, 256, 0, cst>>>(b, d_xyz, s);
-    }
-    const unsigned gp = (unsigned)std::min<long long>((n_pairs + 255) / 256, 152 * 16);
-    k_na_tube<<<gp, 256, 0, cst>>>(b, d_xyz, d_pairs, n_pairs, d_counts, s);
+    const unsigned gc = (unsigned)std::min<long long>((std::max(nx, ny) + 255) / 256, 608);
+    const unsigned gn = (unsigned)std::max<long long>(1, (n + 255) / 256);
+    launch_dep(k_na_clear, dim3(gc), dim3(256), 0, cst, s, (int)nx, (int)ny);
+    launch_dep(k_na_count, dim3(gn), dim3(256), 0, cst, b, d_xyz, s);
+    launch_dep(k_na_scan, dim3(2), dim3(1024), 0, cst, s, (int)nx, (int)ny);
+    launch_dep(k_na_scatter, dim3(gn), dim3(256), 0, cst, b, d_xyz, s);
+    const unsigned gp = (unsigned)std::min<long long>((n_pairs + 4 * NA_W - 1) / (4 * NA_W), 152 * 8);
+    launch_dep(k_na_tube, dim3(gp), dim3(NA_W * 32), 0, cst, b, d_xyz, d_pairs, n_pairs, d_counts, s);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "no-alloc tube count launch");
     return ET_OK;
