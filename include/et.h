@@ -111,8 +111,8 @@ typedef struct {
  * depend on these values, only the speed does. */
 typedef struct {
     int32_t cell[3];        /* cell-list edge per axis, coordinate units; 0: automatic
-                               (s0 * (0.22, 1.1, 1.1), s0 the edge of a cube holding 0.35
-                               grains at the batch's mean density).  The batch's cell table
+                               (s0 * (0.24, 1.75, 1.4), s0 the edge of a cube holding 0.35
+                               grains at the mean density its grains see).  The batch's cell table
                                (views x cells per view) must stay below 2^31 - 1 cells, else
                                loading fails with ET_ERR_INVALID_ARG */
     int32_t ticket_origins; /* origins per work ticket of the seed generator (a warp takes

@@ -26,6 +26,9 @@ enum : u32 {
     ERRB_OVF_MASK = ERRB_OVF_CAND | ERRB_OVF_MEMBERS | ERRB_OVF_RECORD,
 };
 
+// Automatic cell edges, in units of the edge s0 of a cube holding 0.35 grains.
+constexpr double AUTO_CELL[3] = {0.24, 1.75, 1.4};
+
 // Candidate states during the merge.
 enum : unsigned char { CS_UNDECIDED = 0, CS_ACCEPTED = 1, CS_REJECTED = 2 };
 

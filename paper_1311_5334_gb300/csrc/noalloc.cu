@@ -317,9 +317,8 @@ extern "C" et_status et_tube_count_noalloc(const int32_t *d_xyz, int64_t n, cons
     double s0 = std::cbrt(0.35 * vol / (double)std::max<int64_t>(n, 1));
     long long nx = 0, ny = 0;
     for (int tries = 0; tries < 64; ++tries) {
-        static const double f[3] = {0.2, 1.7, 1.4};
         nx = ny = 1;
-        for (int k = 0; k < 3; ++k) b.cs[k] = (int)std::min<double>(std::max(1.0, std::round(s0 * f[k])), b.ext[k]);
+        for (int k = 0; k < 3; ++k) b.cs[k] = (int)std::min<double>(std::max(1.0, std::round(s0 * AUTO_CELL[k])), b.ext[k]);
         b.csy[0] = std::min(b.cs[1], b.ext[0]);
         b.csy[1] = std::min(b.cs[0], b.ext[1]);
         b.csy[2] = b.cs[2];
