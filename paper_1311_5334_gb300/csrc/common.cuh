@@ -29,6 +29,9 @@ enum : u32 {
 // Automatic cell edges, in units of the edge s0 of a cube holding 0.35 grains.
 constexpr double AUTO_CELL[3] = {0.24, 1.75, 1.4};
 
+// Fewest candidates per window of the association, unless set.
+constexpr u64 ASSOC_WINDOW = 1ull << 18;
+
 // Candidate states during the merge.
 enum : unsigned char { CS_UNDECIDED = 0, CS_ACCEPTED = 1, CS_REJECTED = 2 };
 
@@ -38,7 +41,7 @@ struct Ctl {
     u64 n_tests;        // tube tests performed
     u64 n_hits;         // sum of counts over seeds
     u64 n_cand;         // candidates appended (may exceed capacity -> overflow bit)
-    u64 n_members;      // sum of candidate counts (scan result)
+    u64 n_members;      // sum of candidate counts
     u64 n_acc;          // accepted tracks
     u64 n_out_members;  // members of accepted tracks
     u64 n_record;       // per-seed records written (diagnostic path)
@@ -99,7 +102,7 @@ struct Work {
     int *c_lo, *c_hi;    // canonical global indices
     u32 *c_cnt;          // tube count
     u64 *c_key;          // (2^21-1-count) << 42 | rank_lo << 21 | rank_hi
-    u64 *c_moff;         // member offsets, cap + 1
+    u64 *c_moff;         // start of the member list (c_cnt entries)
     unsigned char *c_state;
     u32 *c_nfree;        // unused grains when accepted
     u64 cand_cap;
@@ -109,7 +112,9 @@ struct Work {
     u64 *best[2];        // per grain
     int *owner;          // per grain: accepting candidate or -1
     int *clist[2];       // undecided candidates carried to the next round (cand_cap each)
-    const u32 *corder;   // candidates in key order (the association's windows)
+    const u32 *corder;   // candidates in key order (the association's windows); not read while they are one window
+    u64 *order_k;        // input of the sort into that order (null: no sort)
+    u32 *order_v;
     u64 window;          // candidates per window (0: automatic)
     // diagnostic per-seed record (optional)
     int *rec_lo, *rec_hi, *rec_cnt;
@@ -246,7 +251,8 @@ size_t radix_temp_bytes(long long n);
 // err_bit is already set the sort does nothing.  Every write stays inside
 // [0, n).
 int radix_sort_pairs_dev(u64 *k0, u32 *v0, u64 *k1, u32 *v1, long long n_cap, const u64 *n_dev, int bits,
-                         void *temp, cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit = 0);
+                         void *temp, cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit = 0,
+                         long long n_skip = 0);
 inline int radix_sort_pairs(u64 *k0, u32 *v0, u64 *k1, u32 *v1, long long n, int bits, void *temp,
                             cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit = 0) {
     return radix_sort_pairs_dev(k0, v0, k1, v1, n, nullptr, bits, temp, st, err, err_bit, bar, spin_limit);
@@ -275,12 +281,11 @@ void launch_y_cells(const Batch &b, u32 *cell_of, u32 *cell_count, cudaStream_t 
 
 // count.cu
 void launch_tube_count(const Batch &b, const Work &w, int record, cudaStream_t st);
-// sort_k / sort_v: input of the candidate-order sort (null: not written)
-void launch_cand_keys(const Batch &b, const Work &w, u64 *sort_k, u32 *sort_v, cudaStream_t st);
 void launch_member_fill(const Batch &b, const Work &w, cudaStream_t st);
 void launch_single_pass(const Batch &b, const Work &w, cudaStream_t st);
-// candidates in key order, from the sort input written by launch_cand_keys
-const u32 *launch_cand_order(const Batch &b, const Work &w, Out &o, void *temp, cudaStream_t st);
+// candidates in key order, from the sort input written by the tube counts; nothing is
+// done for at most `window` candidates
+const u32 *launch_cand_order(const Batch &b, const Work &w, Out &o, u64 window, void *temp, cudaStream_t st);
 
 // merge.cu
 int merge_grid_blocks(int device);

@@ -207,6 +207,47 @@ __device__ __forceinline__ bool gen_pass(const Batch &b, GenSm<SG> &sm, GenState
     return true;
 }
 
+// Appends the lanes' accepted seeds (cm: the lanes with is_cand) to the
+// candidates, complete: key (2^21 - 1 - count) << 42 | rank_lo << 21 | rank_hi,
+// whose ascending order is count descending, then ranks ascending; the place of
+// its member list (lists lie in the order the candidates were appended); and
+// the input of the candidate-order sort where there is one.
+__device__ __forceinline__ void append_candidates(const Batch &b, const Work &w, bool is_cand, unsigned cm, int lo,
+                                                  int hi, u32 count, int view) {
+    const int lane = threadIdx.x & 31, leader = __ffs(cm) - 1;
+    u32 incl = is_cand ? count : 0u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const u32 t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const u32 total = __shfl_sync(0xffffffffu, incl, 31);
+    u64 idx = 0, m0 = 0;
+    if (lane == leader) {
+        idx = atomicAdd(&b.ctl->n_cand, (u64)__popc(cm));
+        m0 = atomicAdd(&b.ctl->n_members, (u64)total);
+    }
+    idx = __shfl_sync(0xffffffffu, idx, leader) + __popc(cm & ((1u << lane) - 1u));
+    m0 = __shfl_sync(0xffffffffu, m0, leader) + incl - count;
+    if (!is_cand) return;
+    if (idx >= w.cand_cap) {
+        atomicOr(&b.ctl->error, ERRB_OVF_CAND);
+        return;
+    }
+    const u64 g0 = (u64)b.goff[view];
+    const u64 key = ((((1ull << 21) - 1ull) - count) << 42) | (((u64)lo - g0) << 21) | ((u64)hi - g0);
+    w.c_lo[idx] = lo;
+    w.c_hi[idx] = hi;
+    w.c_cnt[idx] = count;
+    w.c_key[idx] = key;
+    w.c_moff[idx] = m0;
+    w.c_state[idx] = CS_UNDECIDED;
+    if (w.order_k) {
+        w.order_k[idx] = cand_sort_key(b, key);
+        w.order_v[idx] = (u32)idx;
+    }
+}
+
 template <int SG>
 __global__ void __launch_bounds__(TW * 32, 4) k_tube_count(Batch b, Work w, int record) {
     griddep_launch();
@@ -270,22 +311,7 @@ __global__ void __launch_bounds__(TW * 32, 4) k_tube_count(Batch b, Work w, int 
         }
         const bool is_cand = valid && count >= (u32)b.H;
         const unsigned cm = __ballot_sync(0xffffffffu, is_cand);
-        if (cm) {
-            const int leader = __ffs(cm) - 1;
-            u64 base_idx = 0;
-            if (lane == leader) base_idx = atomicAdd(&b.ctl->n_cand, (u64)__popc(cm));
-            base_idx = __shfl_sync(0xffffffffu, base_idx, leader);
-            if (is_cand) {
-                const u64 idx = base_idx + __popc(cm & ((1u << lane) - 1u));
-                if (idx < w.cand_cap) {
-                    w.c_lo[idx] = lo;
-                    w.c_hi[idx] = hi;
-                    w.c_cnt[idx] = count;
-                } else {
-                    atomicOr(&b.ctl->error, ERRB_OVF_CAND);
-                }
-            }
-        }
+        if (cm) append_candidates(b, w, is_cand, cm, lo, hi, count, view);
         __syncwarp();
     }
     const u64 wtests = warp_sum_u64(tests), whits = warp_sum_u64(hits);
@@ -295,32 +321,6 @@ __global__ void __launch_bounds__(TW * 32, 4) k_tube_count(Batch b, Work w, int 
         if (wpairs) atomicAdd(&b.ctl->n_pair_tests, wpairs);
         if (whits) atomicAdd(&b.ctl->n_hits, whits);
         if (nseeds) atomicAdd(&b.ctl->n_seeds, nseeds);
-    }
-}
-
-// Candidate keys: (2^21 - 1 - count) << 42 | rank_lo << 21 | rank_hi, so that
-// ascending keys visit candidates by count descending, then ranks ascending.
-// With sk not null, also the input of the candidate-order sort: the key on
-// 3 * rbits bits and the candidate index.
-__global__ void k_cand_keys(Batch b, Work w, u64 *sk, u32 *sv) {
-    griddep_launch();
-    griddep_wait();
-    if (input_failed(b.ctl)) return;
-    const u64 nc = min(b.ctl->n_cand, w.cand_cap);
-    const u64 stride = (u64)gridDim.x * blockDim.x;
-    for (u64 c = (u64)blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += stride) {
-        const int lo = w.c_lo[c], hi = w.c_hi[c];
-        const int v = view_of(b.goff, b.V, lo);
-        const u64 rlo = (u64)(lo - b.goff[v]), rhi = (u64)(hi - b.goff[v]);
-        const u64 cnt = w.c_cnt[c];
-        const u64 key = ((((1ull << 21) - 1ull) - cnt) << 42) | (rlo << 21) | rhi;
-        w.c_key[c] = key;
-        w.c_moff[c] = cnt;
-        w.c_state[c] = CS_UNDECIDED;
-        if (sk) {
-            sk[c] = cand_sort_key(b, key);
-            sv[c] = (u32)c;
-        }
     }
 }
 
@@ -393,10 +393,6 @@ void launch_tube_count(const Batch &b, const Work &w, int record, cudaStream_t s
     if (b.gen_origins == 1) launch_dep(k_tube_count<1>, dim3(persistent_grid(8)), dim3(TW * 32), 0, st, b, w, record);
     else if (b.gen_origins == 4) launch_dep(k_tube_count<4>, dim3(persistent_grid(8)), dim3(TW * 32), 0, st, b, w, record);
     else launch_dep(k_tube_count<2>, dim3(persistent_grid(8)), dim3(TW * 32), 0, st, b, w, record);
-}
-
-void launch_cand_keys(const Batch &b, const Work &w, u64 *sort_k, u32 *sort_v, cudaStream_t st) {
-    launch_dep(k_cand_keys, dim3(persistent_grid(4)), dim3(256), 0, st, b, w, sort_k, sort_v);
 }
 
 void launch_member_fill(const Batch &b, const Work &w, cudaStream_t st) {

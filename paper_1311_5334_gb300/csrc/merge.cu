@@ -75,7 +75,10 @@ __global__ void __launch_bounds__(MT) k_merge(Batch b, Work w) {
     const u32 H = (u32)b.H;
     __shared__ int keep[MT / 32][32];   // per warp: undecided candidates waiting to be appended
     // candidates per window: at least 2^18, at most 128 windows, unless set
-    const u64 win = w.window ? w.window : max((u64)1 << 18, (nc + 128 - 1) / 128);
+    const u64 win = w.window ? w.window : max(ASSOC_WINDOW, (nc + 128 - 1) / 128);
+    // one window: its rounds give the same result in any order, and the
+    // candidates were not sorted
+    const u32 *corder = nc > win ? w.corder : nullptr;
     u32 round = 0;   // counts all rounds: it selects the ping-pong buffers
     for (u64 w0 = 0; w0 < nc; w0 += win) {
     const u64 w1 = min(nc, w0 + win);
@@ -91,9 +94,9 @@ __global__ void __launch_bounds__(MT) k_merge(Batch b, Work w) {
         u32 my_active = 0;
         for (long long i = gwarp; i < nl; i += nwarps) {
             // lists and states are rewritten by other SMs between rounds: read through L2
-            const long long c = list ? __ldcg(&list[i]) : (long long)w.corder[w0 + i];
+            const long long c = list ? __ldcg(&list[i]) : (corder ? (long long)corder[w0 + i] : i);
             if (__ldcg(&w.c_state[c]) != CS_UNDECIDED) continue;
-            const u64 m0 = w.c_moff[c], m1 = w.c_moff[c + 1];
+            const u64 m0 = w.c_moff[c], m1 = m0 + w.c_cnt[c];
             if (m1 - m0 <= 32) {   // one chunk: member and its state stay in registers
                 const u64 m = m0 + lane;
                 const bool in = m < m1;
@@ -148,9 +151,9 @@ __global__ void __launch_bounds__(MT) k_merge(Batch b, Work w) {
         u64 *next_n = &ctl->ncl[(round + 1) & 1];
         int nkeep = 0;   // warp-uniform
         for (long long i = gwarp; i < nl; i += nwarps) {
-            const long long c = list ? __ldcg(&list[i]) : (long long)w.corder[w0 + i];
+            const long long c = list ? __ldcg(&list[i]) : (corder ? (long long)corder[w0 + i] : i);
             if (__ldcg(&w.c_state[c]) != CS_UNDECIDED) continue;
-            const u64 m0 = w.c_moff[c], m1 = w.c_moff[c + 1];
+            const u64 m0 = w.c_moff[c], m1 = m0 + w.c_cnt[c];
             const u64 key = w.c_key[c];
             if (m1 - m0 <= 32) {   // one chunk: member and its state stay in registers
                 const u64 m = m0 + lane;
@@ -271,7 +274,7 @@ __global__ void k_sp_best(Batch b, Work w) {
     const int lane = threadIdx.x & 31;
     const u64 nw = (u64)gridDim.x * (blockDim.x >> 5);
     for (u64 c = (u64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < nc; c += nw) {
-        const u64 key = w.c_key[c], m0 = w.c_moff[c], m1 = w.c_moff[c + 1];
+        const u64 key = w.c_key[c], m0 = w.c_moff[c], m1 = m0 + w.c_cnt[c];
         for (u64 m = m0 + lane; m < m1; m += 32) atomicMin(&w.best[0][w.members[m]], key);
     }
 }
@@ -286,7 +289,7 @@ __global__ void k_sp_own(Batch b, Work w) {
     const int lane = threadIdx.x & 31;
     const u64 nw = (u64)gridDim.x * (blockDim.x >> 5);
     for (u64 c = (u64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); c < nc; c += nw) {
-        const u64 key = w.c_key[c], m0 = w.c_moff[c], m1 = w.c_moff[c + 1];
+        const u64 key = w.c_key[c], m0 = w.c_moff[c], m1 = m0 + w.c_cnt[c];
         u32 own = 0;
         for (u64 m = m0 + lane; m < m1; m += 32) own += w.best[0][w.members[m]] == key;
         own = __reduce_add_sync(0xffffffffu, own);
@@ -417,7 +420,7 @@ __global__ void k_fit(Batch b, Work w, Out o) {
         const int c = o.acc[t];
         const int lo = w.c_lo[c], hi = w.c_hi[c];
         const int4 ga = b.gr[lo], gb = b.gr[hi];
-        const u64 m0 = w.c_moff[c], m1 = w.c_moff[c + 1];
+        const u64 m0 = w.c_moff[c], m1 = m0 + w.c_cnt[c];
         const u64 obase = o.trk_moff[t];
         long long s1[3] = {0, 0, 0}, s2[6] = {0, 0, 0, 0, 0, 0};
         u32 written = 0;
@@ -557,10 +560,10 @@ cudaError_t launch_merge_coop(const Batch &b, const Work &w, int grid, cudaStrea
     return cudaLaunchCooperativeKernel((const void *)k_merge, dim3(grid), dim3(MT), args, 0, st);
 }
 
-const u32 *launch_cand_order(const Batch &b, const Work &w, Out &o, void *temp, cudaStream_t st) {
+const u32 *launch_cand_order(const Batch &b, const Work &w, Out &o, u64 window, void *temp, cudaStream_t st) {
     const int cur = radix_sort_pairs_dev(o.sort_k[0], o.sort_v[0], o.sort_k[1], o.sort_v[1], (long long)o.acc_cap,
                                          &b.ctl->n_cand, 3 * b.rbits, temp, st, &b.ctl->error, ERRB_TIMEOUT,
-                                         b.ctl->bar, b.spin_limit);
+                                         b.ctl->bar, b.spin_limit, (long long)window);
     return o.sort_v[cur];
 }
 

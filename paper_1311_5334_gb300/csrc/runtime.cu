@@ -342,7 +342,7 @@ size_t BatchRT::lay_group(int k, char *base, DevPtrs &P) const {
         P.c_hi = c.take<int>(cc);
         P.c_cnt = c.take<u32>(cc);
         P.c_key = c.take<u64>(cc);
-        P.c_moff = c.take<u64>(cc + 1);
+        P.c_moff = c.take<u64>(cc);
         P.c_state = c.take<unsigned char>(cc);
         P.c_nfree = c.take<u32>(cc);
         P.clist[0] = c.take<int>(cc);
@@ -663,8 +663,15 @@ Out BatchRT::dev_out() const {
 
 et_status BatchRT::enqueue(cudaStream_t st, bool record) {
     const Batch b = dev_batch();
-    const Work w = dev_work();
+    Work w = dev_work();
     Out o = dev_out();
+    // the association sorts its candidates only where they can fill more than one window
+    const u64 window = tune.assoc_window > 0 ? (u64)tune.assoc_window : ASSOC_WINDOW;
+    const bool sp = (p.flags & ET_FLAG_SINGLE_PASS) != 0;
+    if (!sp && cap_cand > window) {
+        w.order_k = o.sort_k[0];
+        w.order_v = o.sort_v[0];
+    }
     const long long n = N;
     const size_t cells = (size_t)V * (size_t)ncell;
     mark(0, st);
@@ -696,20 +703,16 @@ et_status BatchRT::enqueue(cudaStream_t st, bool record) {
         mark(2, st);
         launch_tube_count(b, w, record ? 1 : 0, st);
         mark(3, st);
-        const bool sp = (p.flags & ET_FLAG_SINGLE_PASS) != 0;
-        launch_cand_keys(b, w, sp ? nullptr : o.sort_k[0], sp ? nullptr : o.sort_v[0], st);
-        exclusive_scan_u64_dev(c_moff, c_moff, (long long)cap_cand, &ctl->n_cand, temp, &ctl->n_members, st,
-                               &ctl->error, ERRB_TIMEOUT, ctl->bar, b.spin_limit);
         launch_member_fill(b, w, st);
         cudaMemsetAsync(best[0], 0xFF, sizeof(u64) * n, st);
         cudaMemsetAsync(best[1], 0xFF, sizeof(u64) * n, st);
         cudaMemsetAsync(owner, 0xFF, sizeof(int) * n, st);
         mark(4, st);
-        if (p.flags & ET_FLAG_SINGLE_PASS) {
+        if (sp) {
             launch_single_pass(b, w, st);
         } else {
             Work wm = w;
-            wm.corder = launch_cand_order(b, w, o, temp, st);
+            wm.corder = launch_cand_order(b, w, o, window, temp, st);
             wm.window = tune.assoc_window > 0 ? (u64)tune.assoc_window : 0;
             cudaError_t e = launch_merge_coop(b, wm, ctx->merge_grid, st);
             if (e != cudaSuccess) return cuda_fail(e, "merge launch");

@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(NT, 1) k_rs_small(u64 *k0, u32 *v0, u64 *k1, u
 
 __global__ void __launch_bounds__(RS_T, 4) k_rs_sort(u64 *k0, u32 *v0, u64 *k1, u32 *v1, long long n_cap,
                                                   const u64 *n_dev, int npass, RsTemp tp, u32 *bar, u32 *err,
-                                                  u32 err_bit, unsigned long long lim) {
+                                                  u32 err_bit, unsigned long long lim, long long n_skip) {
     griddep_launch();
     griddep_wait();
     struct Tiles {   // the tiled passes
@@ -375,6 +375,7 @@ __global__ void __launch_bounds__(RS_T, 4) k_rs_sort(u64 *k0, u32 *v0, u64 *k1, 
     u32 (*wcnt)[256] = sm.l.wcnt;
     if (*(volatile u32 *)err & err_bit) return;
     const long long n = eff_n(n_cap, n_dev);
+    if (n <= n_skip) return;
     if (n <= RS_TILE) {   // one tile: block 0 alone, no waits (uniform: every block read the same count)
         if (blockIdx.x == 0 && n > 0)
             block_sort_small<RS_T>(k0, v0, (npass & 1) ? k1 : k0, (npass & 1) ? v1 : v0, (int)n, npass,
@@ -554,11 +555,13 @@ size_t radix_temp_bytes(long long n) {
 }
 
 int radix_sort_pairs_dev(u64 *k0, u32 *v0, u64 *k1, u32 *v1, long long n_cap, const u64 *n_dev, int bits,
-                         void *temp, cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit) {
+                         void *temp, cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit,
+                         long long n_skip) {
     const unsigned limit = sort_grid_limit();
     const long long ntiles = (n_cap + RS_TILE - 1) / RS_TILE;
     int npass = (bits + 7) / 8;
     if (ntiles == 0 || npass == 0) return 0;
+    if (n_cap <= n_skip) return npass & 1;
     if (n_cap <= RSS_MAX) {   // a short list by capacity: one block, every pass on chip
         if (n_cap <= 256 * 8)
             launch_dep(k_rs_small<256>, dim3(1), dim3(256), rss_smem<256>(), st, k0, v0, k1, v1, n_cap, n_dev, npass, err, err_bit);
@@ -574,7 +577,8 @@ int radix_sort_pairs_dev(u64 *k0, u32 *v0, u64 *k1, u32 *v1, long long n_cap, co
     const unsigned grid = (unsigned)std::min<long long>(ntiles, limit ? (long long)limit : 1ll);
     unsigned long long lim = spin_limit > 0 ? (unsigned long long)spin_limit : (unsigned long long)WAIT_LIMIT;
     void *args[] = {(void *)&k0, (void *)&v0,  (void *)&k1,  (void *)&v1,      (void *)&n_cap, (void *)&n_dev,
-                    (void *)&npass, (void *)&tp, (void *)&bar, (void *)&err, (void *)&err_bit, (void *)&lim};
+                    (void *)&npass, (void *)&tp, (void *)&bar, (void *)&err, (void *)&err_bit, (void *)&lim,
+                    (void *)&n_skip};
     cudaLaunchCooperativeKernel((const void *)k_rs_sort, dim3(grid), dim3(RS_T), args, 0, st);
     return npass & 1;
 }
