@@ -81,17 +81,15 @@ struct Batch {
     const int *xyz_in;   // N x 3 input, caller order
     int4 *gr;            // canonical order: x, y, z, caller index within the view
     int4 *gc;            // cell order: x, y, z, canonical (global) index; the y-row
-                         // list's order follows at gc + N (gcy)
+                         // list's order follows at gc + N
     u64 *gp;             // cell order: x | y << 21 | z << 42 (the tube counts' 8-byte grain loads)
     u32 *cell_start;     // V * ncell + 1
     // second cell list with rows along y: cell edges (cs[1], cs[0], cs[2]),
     // index cy + ncy[1] * (cx + ncy[0] * cz); lines whose |w_y| > |w_x| walk it
-    int dual;            // 1 if the second list is built and used
+    int dual;            // 1 if the second list is built and used (its starts count from N)
     int csy[3], ncy[3];
     float icsy[3];
     int ncelly;
-    int4 *gcy;
-    u64 *gpy;
     u32 *cell_start_y;   // V * ncelly + 1
     Ctl *ctl;
 };
@@ -264,20 +262,19 @@ size_t scan_temp_bytes(long long n);
 // n_dev is null) in one cooperative launch; writes n + 1 outputs (the last =
 // total), and the total to *total_out when total_out is not null.  In place
 // allowed.  bar, err, err_bit and spin_limit as for the sort.
+// out2 (may be null): a second copy of the first n outputs.
 void exclusive_scan_u32(const u32 *in, u32 *out, long long n, void *temp, cudaStream_t st, u32 *err,
-                        u32 err_bit, u32 *bar, long long spin_limit = 0);
+                        u32 err_bit, u32 *bar, long long spin_limit = 0, u32 *out2 = nullptr);
 void exclusive_scan_u64_dev(const u64 *in, u64 *out, long long n_cap, const u64 *n_dev, void *temp,
                             u64 *total_out, cudaStream_t st, u32 *err, u32 err_bit, u32 *bar,
                             long long spin_limit = 0);
 
 // grid.cu
 void launch_canonical_keys(const Batch &b, u64 *keys, u32 *vals, cudaStream_t st);
-void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *cell_of, u32 *cell_count,
+void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y,
                             cudaStream_t st);
-// cell_start: exclusive scan of the counts; cursor: zeroed per-cell counters
-void launch_cell_scatter(const Batch &b, const u32 *cell_of, const u32 *cell_start, u32 *cursor, int ylist,
-                         cudaStream_t st);
-void launch_y_cells(const Batch &b, u32 *cell_of, u32 *cell_count, cudaStream_t st);
+// cursors: the cell starts, which the scatter counts up
+void launch_cell_scatter(const Batch &b, u32 *cursor, u32 *cursor_y, cudaStream_t st);
 
 // count.cu
 void launch_tube_count(const Batch &b, const Work &w, int record, cudaStream_t st);

@@ -7,7 +7,9 @@
 // 3D grid (the paper's 3D hash tables, Section 3 footnote), x fastest, so that
 // a run of cells along x is one contiguous range of grains.  The list is a
 // counting sort: per-cell counts, their exclusive scan (cell starts), and a
-// scatter that takes slots with an atomic cursor per cell.  The order of the
+// scatter that takes slots with an atomic cursor per cell.  The second list
+// (rows along y) is counted, scanned and filled with the first: its cells follow
+// the first list's in one table, so its grains' positions start at N.  The order of the
 // grains inside one cell is therefore arbitrary; no result depends on it
 // (counts, keys and fits are order-independent, member lists are sorted on
 // output).
@@ -37,8 +39,19 @@ __global__ void k_canonical_keys(Batch b, u64 *keys, u32 *vals) {
     }
 }
 
-__global__ void k_canonical_order(Batch b, const u64 *keys, const u32 *vals, u32 *cell_of,
-                                  u32 *cell_count) {
+// Cells of a grain in the two lists.
+__device__ __forceinline__ u32 cell_x(const Batch &b, int v, int x, int y, int z) {
+    const int cx = min(x / b.cs[0], b.nc[0] - 1), cy = min(y / b.cs[1], b.nc[1] - 1), cz = min(z / b.cs[2], b.nc[2] - 1);
+    return (u32)v * (u32)b.ncell + (u32)(cx + b.nc[0] * (cy + b.nc[1] * cz));
+}
+__device__ __forceinline__ u32 cell_y(const Batch &b, int v, int x, int y, int z) {
+    const int cx = min(x / b.csy[0], b.ncy[0] - 1), cy = min(y / b.csy[1], b.ncy[1] - 1);
+    const int cz = min(z / b.csy[2], b.ncy[2] - 1);
+    return (u32)v * (u32)b.ncelly + (u32)(cy + b.ncy[1] * (cx + b.ncy[0] * cz));
+}
+
+// Grains into canonical order, and the counts of their cells in both lists.
+__global__ void k_canonical_order(Batch b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y) {
     griddep_launch();
     griddep_wait();
     // a coordinate out of range is reported as such; a timed-out sort leaves
@@ -54,34 +67,15 @@ __global__ void k_canonical_order(Batch b, const u64 *keys, const u32 *vals, u32
         z = min(max(z, 0), b.ext[2] - 1);
         b.gr[p] = make_int4(x, y, z, (int)(i - b.goff[v]));
         if (p > b.goff[v] && keys[p] == keys[p - 1]) atomicOr(&b.ctl->error, ERRB_DUPLICATE);
-        int cx = min(x / b.cs[0], b.nc[0] - 1);
-        int cy = min(y / b.cs[1], b.nc[1] - 1);
-        int cz = min(z / b.cs[2], b.nc[2] - 1);
-        u32 cell = (u32)v * (u32)b.ncell + (u32)(cx + b.nc[0] * (cy + b.nc[1] * cz));
-        cell_of[p] = cell;
-        atomicAdd(&cell_count[cell], 1u);
+        atomicAdd(&count[cell_x(b, v, x, y, z)], 1u);
+        if (b.dual) atomicAdd(&count_y[cell_y(b, v, x, y, z)], 1u);
     }
 }
 
-// Scatter of the canonical order into a cell list: grain p takes the next
-// slot of its cell (cursor zeroed before the launch).
-__global__ void k_cell_scatter(Batch b, const u32 *cell_of, const u32 *cell_start, u32 *cursor, int4 *gc,
-                               u64 *gp) {
-    griddep_launch();
-    griddep_wait();
-    if (input_failed(b.ctl)) return;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < b.N; p += stride) {
-        const u32 c = cell_of[p];
-        const u32 q = cell_start[c] + atomicAdd(&cursor[c], 1u);
-        const int4 g = b.gr[p];
-        gc[q] = make_int4(g.x, g.y, g.z, (int)p);
-        gp[q] = pack_xyz(g.x, g.y, g.z);
-    }
-}
-
-// Cells of the second cell list (rows along y) for the canonical order.
-__global__ void k_y_cells(Batch b, u32 *cell_of, u32 *cell_count) {
+// Scatter of the canonical order into the cell lists: a grain takes the next
+// slot of its cells (the cursors begin as the cell starts; the y-row list's
+// positions begin at N).
+__global__ void k_cell_scatter(Batch b, u32 *cursor, u32 *cursor_y) {
     griddep_launch();
     griddep_wait();
     if (input_failed(b.ctl)) return;
@@ -89,12 +83,14 @@ __global__ void k_y_cells(Batch b, u32 *cell_of, u32 *cell_count) {
     for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < b.N; p += stride) {
         const int v = view_of(b.goff, b.V, p);
         const int4 g = b.gr[p];
-        const int cx = min(g.x / b.csy[0], b.ncy[0] - 1);
-        const int cy = min(g.y / b.csy[1], b.ncy[1] - 1);
-        const int cz = min(g.z / b.csy[2], b.ncy[2] - 1);
-        const u32 cell = (u32)v * (u32)b.ncelly + (u32)(cy + b.ncy[1] * (cx + b.ncy[0] * cz));
-        cell_of[p] = cell;
-        atomicAdd(&cell_count[cell], 1u);
+        const u32 q = atomicAdd(&cursor[cell_x(b, v, g.x, g.y, g.z)], 1u);
+        b.gc[q] = make_int4(g.x, g.y, g.z, (int)p);
+        b.gp[q] = pack_xyz(g.x, g.y, g.z);
+        if (b.dual) {
+            const u32 qy = atomicAdd(&cursor_y[cell_y(b, v, g.x, g.y, g.z)], 1u);
+            b.gc[qy] = make_int4(g.x, g.y, g.z, (int)p);
+            b.gp[qy] = pack_xyz(g.x, g.y, g.z);
+        }
     }
 }
 
@@ -111,19 +107,13 @@ void launch_canonical_keys(const Batch &b, u64 *keys, u32 *vals, cudaStream_t st
     launch_dep(k_canonical_keys, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, keys, vals);
 }
 
-void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *cell_of, u32 *cell_count,
+void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y,
                             cudaStream_t st) {
-    launch_dep(k_canonical_order, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, keys, vals, cell_of, cell_count);
+    launch_dep(k_canonical_order, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, keys, vals, count, count_y);
 }
 
-void launch_cell_scatter(const Batch &b, const u32 *cell_of, const u32 *cell_start, u32 *cursor, int ylist,
-                         cudaStream_t st) {
-    launch_dep(k_cell_scatter, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, cell_of, cell_start, cursor, ylist ? b.gcy : b.gc,
-                                                       ylist ? b.gpy : b.gp);
-}
-
-void launch_y_cells(const Batch &b, u32 *cell_of, u32 *cell_count, cudaStream_t st) {
-    launch_dep(k_y_cells, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, cell_of, cell_count);
+void launch_cell_scatter(const Batch &b, u32 *cursor, u32 *cursor_y, cudaStream_t st) {
+    launch_dep(k_cell_scatter, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, cursor, cursor_y);
 }
 
 }  // namespace et

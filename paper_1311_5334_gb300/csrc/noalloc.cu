@@ -115,13 +115,13 @@ __global__ void k_na_count(Batch b, const int *xyz, NaScratch s) {
 // one-thread-per-cell shared-memory scan of one list took 53 us.
 constexpr int NA_SC = 8;
 
-__global__ void __launch_bounds__(1024) k_na_scan(NaScratch s, int n0, int n1) {
+__global__ void __launch_bounds__(1024) k_na_scan(NaScratch s, int n0, int n1, u32 N) {
     griddep_launch();
     griddep_wait();
     __shared__ u32 part[32];
     const int list = blockIdx.x, n = list ? n1 : n0, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     u32 *cur = s.cursor[list], *start = s.start[list];
-    u32 carry = 0, v[NA_SC], next[NA_SC];
+    u32 carry = list ? N : 0u, v[NA_SC], next[NA_SC];   // the second list lies behind N
     auto load = [&](int base, u32 (&d)[NA_SC]) {
         const int c = base + (int)threadIdx.x * NA_SC;
 #pragma unroll
@@ -175,7 +175,7 @@ __global__ void k_na_scatter(Batch b, const int *xyz, NaScratch s) {
         if (!na_inside(b, x, y, z)) continue;
         const u64 g = pack_xyz(x, y, z);
         s.grains[atomicAdd(&s.cursor[0][na_cell_x(b, x, y, z)], 1u)] = g;
-        s.grains[(u32)b.N + atomicAdd(&s.cursor[1][na_cell_y(b, x, y, z)], 1u)] = g;
+        s.grains[atomicAdd(&s.cursor[1][na_cell_y(b, x, y, z)], 1u)] = g;
     }
 }
 
@@ -346,7 +346,7 @@ extern "C" et_status et_tube_count_noalloc(const int32_t *d_xyz, int64_t n, cons
     const unsigned gn = (unsigned)std::max<long long>(1, (n + 255) / 256);
     launch_dep(k_na_clear, dim3(gc), dim3(256), 0, cst, s, (int)nx, (int)ny);
     launch_dep(k_na_count, dim3(gn), dim3(256), 0, cst, b, d_xyz, s);
-    launch_dep(k_na_scan, dim3(2), dim3(1024), 0, cst, s, (int)nx, (int)ny);
+    launch_dep(k_na_scan, dim3(2), dim3(1024), 0, cst, s, (int)nx, (int)ny, (u32)n);
     launch_dep(k_na_scatter, dim3(gn), dim3(256), 0, cst, b, d_xyz, s);
     const unsigned gp = (unsigned)std::min<long long>((n_pairs + 4 * NA_W - 1) / (4 * NA_W), 152 * 8);
     launch_dep(k_na_tube, dim3(gp), dim3(NA_W * 32), 0, cst, b, d_xyz, d_pairs, n_pairs, d_counts, s);

@@ -281,11 +281,11 @@ struct DevPtrs {
     int *xyz_in = nullptr;
     u64 *keys[2] = {nullptr, nullptr};
     u32 *vals[2] = {nullptr, nullptr};
-    int4 *gr = nullptr, *gc = nullptr, *gcy = nullptr;
-    u64 *gp = nullptr, *gpy = nullptr;
+    int4 *gr = nullptr, *gc = nullptr;
+    u64 *gp = nullptr;
     u64 *best[2] = {nullptr, nullptr};
     int *owner = nullptr;
-    u32 *cell_count = nullptr, *cell_start = nullptr, *cell_count_y = nullptr, *cell_start_y = nullptr;
+    u32 *cell_count = nullptr, *cell_start = nullptr;
     int *c_lo = nullptr, *c_hi = nullptr;
     u32 *c_cnt = nullptr, *c_nfree = nullptr;
     u64 *c_key = nullptr, *c_moff = nullptr;
@@ -306,7 +306,7 @@ struct DevPtrs {
 size_t BatchRT::lay_group(int k, char *base, DevPtrs &P) const {
     Carver c{0, base};
     const size_t n = (size_t)std::max<long long>(N, 1);
-    const size_t cells = (size_t)V * (size_t)ncell, cellsy = (size_t)V * (size_t)ncelly;
+    const size_t cells = (size_t)V * (size_t)ncell, cellsy = dual ? (size_t)V * (size_t)ncelly : 0;
     switch (k) {
     case 0:   // control block, goff, per-view track offsets
         P.ctl = c.take<Ctl>(1);
@@ -323,18 +323,15 @@ size_t BatchRT::lay_group(int k, char *base, DevPtrs &P) const {
         // the two cell orders back to back (the y-row list at offset n), so a
         // walk addresses either through one array
         P.gc = c.take<int4>(2 * n);
-        P.gcy = P.gc ? P.gc + n : nullptr;
         P.gp = c.take<u64>(2 * n);
-        P.gpy = P.gp ? P.gp + n : nullptr;
         P.best[0] = c.take<u64>(n);
         P.best[1] = c.take<u64>(n);
         P.owner = c.take<int>(n);
         break;
     case 2:
-        P.cell_count = c.take<u32>(cells);
-        P.cell_start = c.take<u32>(cells + 1);
-        P.cell_count_y = c.take<u32>(cellsy);
-        P.cell_start_y = c.take<u32>(cellsy + 1);
+        // the y-row list's cells follow the x-row list's
+        P.cell_count = c.take<u32>(cells + cellsy);
+        P.cell_start = c.take<u32>(cells + cellsy + 1);
         break;
     case 3: {
         const size_t cc = want_cand;
@@ -376,7 +373,7 @@ size_t BatchRT::lay_group(int k, char *base, DevPtrs &P) const {
         size_t t = 0;
         t = std::max(t, radix_temp_bytes((long long)n));
         t = std::max(t, radix_temp_bytes((long long)std::max<size_t>(want_cand, n)));
-        t = std::max(t, scan_temp_bytes((long long)std::max(cells, cellsy) + 1));
+        t = std::max(t, scan_temp_bytes((long long)(cells + cellsy) + 1));
         t = std::max(t, scan_temp_bytes((long long)n + 1));
         t = std::max(t, scan_temp_bytes((long long)want_cand + 1));
         t = std::max(t, scan_temp_bytes((long long)V + 1));
@@ -439,16 +436,12 @@ et_status BatchRT::reserve() {
     vals[1] = P.vals[1];
     gr = P.gr;
     gc = P.gc;
-    gcy = P.gcy;
     gp = P.gp;
-    gpy = P.gpy;
     best[0] = P.best[0];
     best[1] = P.best[1];
     owner = P.owner;
     cell_count = P.cell_count;
     cell_start = P.cell_start;
-    cell_count_y = P.cell_count_y;
-    cell_start_y = P.cell_start_y;
     c_lo = P.c_lo;
     c_hi = P.c_hi;
     c_cnt = P.c_cnt;
@@ -604,9 +597,7 @@ Batch BatchRT::dev_batch() const {
     }
     b.ncelly = (int)ncelly;
     b.dual = dual ? 1 : 0;
-    b.gcy = gcy;
-    b.gpy = gpy;
-    b.cell_start_y = cell_start_y;
+    b.cell_start_y = cell_start + (size_t)V * (size_t)ncell;
     b.vshift = cbits[0] + cbits[1] + cbits[2];
     b.rbits = std::max(1, bits_for((unsigned long long)maxN));
     b.xyz_in = xyz_in;
@@ -673,32 +664,21 @@ et_status BatchRT::enqueue(cudaStream_t st, bool record) {
         w.order_v = o.sort_v[0];
     }
     const long long n = N;
-    const size_t cells = (size_t)V * (size_t)ncell;
+    const size_t cells = (size_t)V * (size_t)ncell, cellsy = dual ? (size_t)V * (size_t)ncelly : 0;
     mark(0, st);
     cudaMemsetAsync(ctl, 0, sizeof(Ctl), st);
     if (n > 0) {
-        cudaMemsetAsync(cell_count, 0, sizeof(u32) * cells, st);
+        cudaMemsetAsync(cell_count, 0, sizeof(u32) * (cells + cellsy), st);
         launch_canonical_keys(b, keys[0], vals[0], st);
         const int kb = b.vshift + bits_for((unsigned long long)std::max(V - 1, 0));
         int c1 = radix_sort_pairs(keys[0], vals[0], keys[1], vals[1], n, kb, temp, st, &ctl->error, ERRB_TIMEOUT,
                                   ctl->bar, b.spin_limit);
-        u32 *sv = vals[c1], *cell_of = vals[c1 ^ 1];
-        launch_canonical_order(b, keys[c1], sv, cell_of, cell_count, st);
-        // cell list by counting sort: starts from the counts, then the counts
-        // are zeroed and serve as per-cell cursors of the scatter
-        exclusive_scan_u32(cell_count, cell_start, (long long)cells, temp, st, &ctl->error, ERRB_TIMEOUT, ctl->bar,
-                           b.spin_limit);
-        cudaMemsetAsync(cell_count, 0, sizeof(u32) * cells, st);
-        launch_cell_scatter(b, cell_of, cell_start, cell_count, 0, st);
-        if (dual) {   // second cell list (rows along y) from the same canonical order
-            const size_t cellsy = (size_t)V * (size_t)ncelly;
-            cudaMemsetAsync(cell_count_y, 0, sizeof(u32) * cellsy, st);
-            launch_y_cells(b, cell_of, cell_count_y, st);
-            exclusive_scan_u32(cell_count_y, cell_start_y, (long long)cellsy, temp, st, &ctl->error, ERRB_TIMEOUT,
-                               ctl->bar, b.spin_limit);
-            cudaMemsetAsync(cell_count_y, 0, sizeof(u32) * cellsy, st);
-            launch_cell_scatter(b, cell_of, cell_start_y, cell_count_y, 1, st);
-        }
+        launch_canonical_order(b, keys[c1], vals[c1], cell_count, cell_count + cells, st);
+        // both cell lists by one counting sort: the scan leaves the starts, and in
+        // the counts' place a copy that serves as the scatter's cursors
+        exclusive_scan_u32(cell_count, cell_start, (long long)(cells + cellsy), temp, st, &ctl->error, ERRB_TIMEOUT,
+                           ctl->bar, b.spin_limit, cell_count);
+        launch_cell_scatter(b, cell_count, cell_count + cells, st);
         mark(1, st);   // seeds are generated inside the tube-count kernel: stage 1 stays empty
         mark(2, st);
         launch_tube_count(b, w, record ? 1 : 0, st);

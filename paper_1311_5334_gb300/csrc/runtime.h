@@ -81,13 +81,11 @@ struct BatchRT {
     u64 *keys[2] = {nullptr, nullptr};
     u32 *vals[2] = {nullptr, nullptr};
     int4 *gr = nullptr, *gc = nullptr;
-    u64 *gp = nullptr, *gpy = nullptr;
+    u64 *gp = nullptr;
     u64 *best[2] = {nullptr, nullptr};
     int *owner = nullptr;
     int *clist[2] = {nullptr, nullptr};
     u32 *cell_count = nullptr, *cell_start = nullptr;
-    u32 *cell_count_y = nullptr, *cell_start_y = nullptr;
-    int4 *gcy = nullptr;
     int *c_lo = nullptr, *c_hi = nullptr;
     u32 *c_cnt = nullptr, *c_nfree = nullptr;
     u64 *c_key = nullptr, *c_moff = nullptr;

@@ -82,7 +82,7 @@ __device__ __forceinline__ long long eff_n(long long n_cap, const u64 *n_dev) {
 // own.  Then every block scans its run tile by tile with a running carry; the
 // last block writes the total.
 template <class T>
-__global__ void __launch_bounds__(SC_T) k_scan(const T *in, T *out, long long n_cap, const u64 *n_dev, T *partial,
+__global__ void __launch_bounds__(SC_T) k_scan(const T *in, T *out, T *out2, long long n_cap, const u64 *n_dev, T *partial,
                                                u64 *total_out, u32 *bar, u32 *err, u32 err_bit,
                                                unsigned long long lim) {
     griddep_launch();
@@ -124,7 +124,10 @@ __global__ void __launch_bounds__(SC_T) k_scan(const T *in, T *out, long long n_
         T ex = block_excl_scan(s, tot) + carry;
 #pragma unroll
         for (int i = 0; i < SC_I; ++i) {
-            if (base + i < n) out[base + i] = ex;
+            if (base + i < n) {
+                out[base + i] = ex;
+                if (out2) out2[base + i] = ex;
+            }
             ex += v[i];
         }
         carry += tot;
@@ -142,7 +145,7 @@ unsigned scan_grid_limit() {
 }
 
 template <class T>
-void scan_impl(const T *in, T *out, long long n_cap, const u64 *n_dev, void *temp, u64 *total_out,
+void scan_impl(const T *in, T *out, T *out2, long long n_cap, const u64 *n_dev, void *temp, u64 *total_out,
                cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit) {
     const unsigned limit = scan_grid_limit<T>();
     long long nt = (n_cap + SC_TILE - 1) / SC_TILE;
@@ -150,7 +153,7 @@ void scan_impl(const T *in, T *out, long long n_cap, const u64 *n_dev, void *tem
     unsigned grid = (unsigned)std::min<long long>(nt, limit ? (long long)limit : 1ll);
     T *partial = (T *)temp;
     unsigned long long lim = spin_limit > 0 ? (unsigned long long)spin_limit : (unsigned long long)WAIT_LIMIT;
-    void *args[] = {(void *)&in, (void *)&out, (void *)&n_cap, (void *)&n_dev, (void *)&partial,
+    void *args[] = {(void *)&in, (void *)&out, (void *)&out2, (void *)&n_cap, (void *)&n_dev, (void *)&partial,
                     (void *)&total_out, (void *)&bar, (void *)&err, (void *)&err_bit, (void *)&lim};
     cudaLaunchCooperativeKernel((const void *)k_scan<T>, dim3(grid), dim3(SC_T), args, 0, st);
 }
@@ -539,13 +542,13 @@ size_t scan_temp_bytes(long long n) {
 }
 
 void exclusive_scan_u32(const u32 *in, u32 *out, long long n, void *temp, cudaStream_t st, u32 *err, u32 err_bit,
-                        u32 *bar, long long spin_limit) {
-    scan_impl<u32>(in, out, n, nullptr, temp, nullptr, st, err, err_bit, bar, spin_limit);
+                        u32 *bar, long long spin_limit, u32 *out2) {
+    scan_impl<u32>(in, out, out2, n, nullptr, temp, nullptr, st, err, err_bit, bar, spin_limit);
 }
 
 void exclusive_scan_u64_dev(const u64 *in, u64 *out, long long n_cap, const u64 *n_dev, void *temp,
                             u64 *total_out, cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit) {
-    scan_impl<u64>(in, out, n_cap, n_dev, temp, total_out, st, err, err_bit, bar, spin_limit);
+    scan_impl<u64>(in, out, nullptr, n_cap, n_dev, temp, total_out, st, err, err_bit, bar, spin_limit);
 }
 
 size_t radix_temp_bytes(long long n) {

@@ -217,7 +217,6 @@ __device__ __forceinline__ void warp_items(const Batch &b, SeedTab &sp, int4 *tb
         const int own = before + __popc(smask & lane_le) - 1;
         const int item = ibase + lane;
         u32 b0 = 0, n0 = 0, b1 = 0, n1 = 0;
-        u32 loff = 0;   // N for the y-row list (its cell order follows the x-row one)
         if (item < total) {
             const float4 e2 = sp.f4(2, own), e3 = sp.f4(3, own);
             const int co = __float_as_int(e2.z) + (item - __float_as_int(e2.w));
@@ -228,7 +227,6 @@ __device__ __forceinline__ void warp_items(const Batch &b, SeedTab &sp, int4 *tb
                 const int4 e7 = sp.i4(7, own);
                 const int flags = __float_as_int(e5.w);
                 const int list = flags & 1;
-                loff = list ? (u32)b.N : 0u;
                 const bool ineg = (flags & 2) != 0, rneg = (flags & 4) != 0;
                 // inner cells reached over [ta, tb]
                 const float il = fmaf(ineg ? tb : ta, e5.z, e5.x), ih = fmaf(ineg ? ta : tb, e5.z, e5.y);
@@ -286,7 +284,7 @@ __device__ __forceinline__ void warp_items(const Batch &b, SeedTab &sp, int4 *tb
                             (long long)(((unsigned long long)(unsigned)e1.w << 32) | (unsigned)e1.z);
                         tests += end - beg;
                         for (u32 k = beg; k < end; ++k) {
-                            const int4 g = grain_at<PACKED>(b, loff + k);
+                            const int4 g = grain_at<PACKED>(b, k);
                             if (in_tube(g, a, d, R)) hit(own, g);
                         }
                     }
@@ -306,7 +304,7 @@ __device__ __forceinline__ void warp_items(const Batch &b, SeedTab &sp, int4 *tb
 #pragma unroll
                 for (int j = 0; j < SERIAL; ++j) {
                     if ((u32)j < s0 + s1) {
-                        const u32 k = loff + ((u32)j < s0 ? b0 + (u32)j : b1 + ((u32)j - s0));
+                        const u32 k = (u32)j < s0 ? b0 + (u32)j : b1 + ((u32)j - s0);
                         const int4 g = grain_at<PACKED>(b, k);
                         const bool h = in_tube(g, a, d, R);
                         if (COUNT) red_add_if(h, &cnt[own]);
@@ -330,9 +328,9 @@ __device__ __forceinline__ void warp_items(const Batch &b, SeedTab &sp, int4 *tb
         const u32 rtotal = __shfl_sync(0xffffffffu, rin, 31);
         const u32 rex = rin - n;
         const unsigned nonempty = __ballot_sync(0xffffffffu, n > 0);
-        if (n > 0)   // offsets into the two lists back to back
+        if (n > 0)
             tbl[__popc(nonempty & lane_lt)] =
-                make_int4((int)(b0 + loff - rex), (int)(rex + n0), (int)(b1 + loff - rex - n0), own);
+                make_int4((int)(b0 - rex), (int)(rex + n0), (int)(b1 - rex - n0), own);
         __syncwarp();
         // two passes per iteration, so that their table, geometry and grain
         // loads overlap; a last part of at most 32 grains takes one pass
