@@ -53,6 +53,7 @@ struct Ctl {
     u64 ncl[2];         // merge: lengths of the undecided-candidate lists (ping-pong)
     u32 round_active[64];   // merge: participants of the first 64 rounds (diagnostics)
     u64 ticket[2];          // work tickets of the tube-count and member-list kernels
+    u32 n_long, pad2;       // tracks in Out::long_tracks
     u64 n_pair_tests;       // seed-window tests of the seed generator
 };
 
@@ -130,7 +131,7 @@ struct Out {
     long long *view_trk; // V + 1 track offsets
     void *tracks;        // et_track[acc_cap]
     int *out_members;    // caller indices, sorted within each track
-    u64 out_member_cap;
+    int *long_tracks;    // tracks whose members are sorted on their own
 };
 
 __device__ __forceinline__ int view_of(const long long *goff, int V, long long g) {

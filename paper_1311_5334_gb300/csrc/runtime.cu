@@ -13,8 +13,7 @@
 namespace et {
 
 cudaError_t launch_merge_coop(const Batch &b, const Work &w, int grid, cudaStream_t st);
-void launch_output(const Batch &b, const Work &w, Out &o, long long acc_cap, long long out_member_cap,
-                   void *temp, cudaStream_t st);
+void launch_output(const Batch &b, const Work &w, Out &o, long long acc_cap, void *temp, cudaStream_t st);
 
 static thread_local std::string g_last_error;
 
@@ -648,7 +647,7 @@ Out BatchRT::dev_out() const {
     o.view_trk = view_trk;
     o.tracks = tracks;
     o.out_members = out_members;
-    o.out_member_cap = (u64)std::max<long long>(N, 1);
+    o.long_tracks = (int *)sort_v[0];   // idle once the accepted list is in order
     return o;
 }
 
@@ -698,7 +697,7 @@ et_status BatchRT::enqueue(cudaStream_t st, bool record) {
             if (e != cudaSuccess) return cuda_fail(e, "merge launch");
         }
         mark(5, st);
-        launch_output(b, w, o, (long long)cap_cand, std::max<long long>(n, 1), temp, st);
+        launch_output(b, w, o, (long long)cap_cand, temp, st);
         mark(6, st);
     } else {
         cudaMemsetAsync(view_trk, 0, sizeof(long long) * (V + 1), st);
