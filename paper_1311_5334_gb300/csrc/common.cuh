@@ -104,6 +104,7 @@ struct Work {
     u64 *c_moff;         // start of the member list (c_cnt entries)
     unsigned char *c_state;
     u32 *c_nfree;        // unused grains when accepted
+    int *acc;            // accepted candidates in any order (Ctl::n_acc of them)
     u64 cand_cap;
     int *members;        // canonical global indices
     u64 member_cap;

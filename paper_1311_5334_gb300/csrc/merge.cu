@@ -61,7 +61,31 @@ __device__ __forceinline__ u32 ld_cg_u32(const u32 *p) { return __ldcg(p); }
 // cheap, a long one on the whole grid.
 constexpr u64 MERGE_CANDS_PER_BLOCK = MT / 32;
 
-__global__ void __launch_bounds__(MT) k_merge(Batch b, Work w) {
+// Angle cut (ET_FLAG_ANGLE_CUT): keep a track iff
+//     nhits >= cut_base + cut_slope * min(tan theta, cut_tmax),
+// tan theta = sqrt(wx^2 + wy^2) / |wz| for the seed vector w, in exact
+// integers: with A = nhits - cut_base, keep iff A >= 0 and either
+// wx^2 + wy^2 >= cut_tmax^2 wz^2 (tan theta capped) and A >= cut_slope cut_tmax,
+// or A^2 wz^2 >= cut_slope^2 (wx^2 + wy^2) (128-bit products).
+__device__ __forceinline__ bool angle_cut_keeps(const Batch &b, int4 glo, int4 ghi, long long nhits) {
+    const long long A = nhits - b.cut_base;
+    if (A < 0) return false;
+    const long long wx = ghi.x - glo.x, wy = ghi.y - glo.y, wz = ghi.z - glo.z;
+    const unsigned long long t2 = (unsigned long long)(wx * wx + wy * wy), z2 = (unsigned long long)(wz * wz);
+    const unsigned long long tm = (unsigned long long)b.cut_tmax, sl = (unsigned long long)b.cut_slope;
+    if ((unsigned __int128)t2 >= (unsigned __int128)(tm * tm) * z2) return (unsigned long long)A >= sl * tm;
+    return (unsigned __int128)((unsigned long long)A * (unsigned long long)A) * z2 >=
+           (unsigned __int128)(sl * sl) * t2;
+}
+
+// Puts an accepted candidate on the list of tracks (any order), unless the
+// angle cut drops it.
+__device__ __forceinline__ void take_track(const Batch &b, const Work &w, long long c, u32 nfree) {
+    if ((b.flags & ET_FLAG_ANGLE_CUT) && !angle_cut_keeps(b, b.gr[w.c_lo[c]], b.gr[w.c_hi[c]], nfree)) return;
+    w.acc[atomicAdd(&b.ctl->n_acc, 1ull)] = (int)c;
+}
+
+__global__ void __launch_bounds__(MT, 4) k_merge(Batch b, Work w) {
     griddep_launch();
     griddep_wait();
     Ctl *ctl = b.ctl;
@@ -185,6 +209,7 @@ __global__ void __launch_bounds__(MT) k_merge(Batch b, Work w) {
                 if (lane == 0) {
                     w.c_nfree[c] = nfree;
                     w.c_state[c] = accept ? CS_ACCEPTED : CS_REJECTED;
+                    if (accept) take_track(b, w, c, nfree);
                 }
                 continue;
             }
@@ -233,6 +258,7 @@ __global__ void __launch_bounds__(MT) k_merge(Batch b, Work w) {
             if (lane == 0) {
                 w.c_nfree[c] = nfree;
                 w.c_state[c] = accept ? CS_ACCEPTED : CS_REJECTED;
+                if (accept) take_track(b, w, c, nfree);
             }
         }
         if (nkeep > 0) {
@@ -247,23 +273,6 @@ __global__ void __launch_bounds__(MT) k_merge(Batch b, Work w) {
     }
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->rounds = round;
-}
-
-// Angle cut (ET_FLAG_ANGLE_CUT): keep a track iff
-//     nhits >= cut_base + cut_slope * min(tan theta, cut_tmax),
-// tan theta = sqrt(wx^2 + wy^2) / |wz| for the seed vector w, in exact
-// integers: with A = nhits - cut_base, keep iff A >= 0 and either
-// wx^2 + wy^2 >= cut_tmax^2 wz^2 (tan theta capped) and A >= cut_slope cut_tmax,
-// or A^2 wz^2 >= cut_slope^2 (wx^2 + wy^2) (128-bit products).
-__device__ __forceinline__ bool angle_cut_keeps(const Batch &b, int4 glo, int4 ghi, long long nhits) {
-    const long long A = nhits - b.cut_base;
-    if (A < 0) return false;
-    const long long wx = ghi.x - glo.x, wy = ghi.y - glo.y, wz = ghi.z - glo.z;
-    const unsigned long long t2 = (unsigned long long)(wx * wx + wy * wy), z2 = (unsigned long long)(wz * wz);
-    const unsigned long long tm = (unsigned long long)b.cut_tmax, sl = (unsigned long long)b.cut_slope;
-    if ((unsigned __int128)t2 >= (unsigned __int128)(tm * tm) * z2) return (unsigned long long)A >= sl * tm;
-    return (unsigned __int128)((unsigned long long)A * (unsigned long long)A) * z2 >=
-           (unsigned __int128)(sl * sl) * t2;
 }
 
 // Single-pass association (ET_FLAG_SINGLE_PASS), step 1: every grain keeps the
@@ -304,24 +313,114 @@ __global__ void k_sp_own(Batch b, Work w) {
         if (lane == 0) {
             w.c_nfree[c] = own;
             w.c_state[c] = accept ? CS_ACCEPTED : CS_REJECTED;
+            if (accept) take_track(b, w, (long long)c, own);
         }
     }
 }
 
-// Accepted candidates -> list (any order) with sort keys.
-__global__ void k_collect(Batch b, Work w, Out o) {
+// Accepted candidates -> input of the sort into key order.
+__global__ void k_acc_keys(Batch b, Work w, Out o) {
     griddep_launch();
     griddep_wait();
     if (input_failed(b.ctl)) return;
-    const u64 nc = min(b.ctl->n_cand, w.cand_cap);
+    const u64 na = b.ctl->n_acc;
     const u64 stride = (u64)gridDim.x * blockDim.x;
-    for (u64 c = (u64)blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += stride) {
-        if (w.c_state[c] != CS_ACCEPTED) continue;
-        if ((b.flags & ET_FLAG_ANGLE_CUT) && !angle_cut_keeps(b, b.gr[w.c_lo[c]], b.gr[w.c_hi[c]], w.c_nfree[c]))
-            continue;
-        const u64 i = atomicAdd(&b.ctl->n_acc, 1ull);
+    for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < na; i += stride) {
+        const int c = w.acc[i];
         o.sort_k[0][i] = cand_sort_key(b, w.c_key[c]);
         o.sort_v[0][i] = (u32)c;
+    }
+}
+
+// The whole order of at most ACC_SMALL accepted tracks in one block: (view,
+// key) sorted by a bitonic network in shared memory, then their views, member
+// offsets and the views' track offsets.  It replaces five launches (eight with
+// more than one view) of the general path below, each a few us on one view.
+constexpr int ACC_T = 1024, ACC_SMALL = 4096;
+
+__global__ void __launch_bounds__(ACC_T) k_acc_small(Batch b, Work w, Out o) {
+    griddep_launch();
+    griddep_wait();
+    if (input_failed(b.ctl)) return;
+    extern __shared__ __align__(16) u64 acc_smem[];
+    u64 *key = acc_smem;
+    u32 *val = (u32 *)(acc_smem + ACC_SMALL);
+    __shared__ u32 wsum[ACC_T / 32];
+    const int t = threadIdx.x, lane = t & 31, wib = t >> 5, kb = 3 * b.rbits;
+    const int n = (int)min(b.ctl->n_acc, (u64)ACC_SMALL);
+    int n2 = 32;
+    while (n2 < n) n2 *= 2;
+    for (int i = t; i < n2; i += ACC_T) {
+        u64 k = ~0ull;
+        u32 c = 0;
+        if (i < n) {
+            c = (u32)w.acc[i];
+            k = cand_sort_key(b, w.c_key[c]);
+            if (b.V > 1) k |= (u64)view_of(b.goff, b.V, w.c_lo[c]) << kb;
+        }
+        key[i] = k;
+        val[i] = c;
+    }
+    __syncthreads();
+    for (int size = 2; size <= n2; size *= 2)
+        for (int step = size / 2; step > 0; step /= 2) {
+            for (int i = t; i < n2 / 2; i += ACC_T) {
+                const int x = 2 * i - (i & (step - 1)), y = x + step;
+                const bool up = (x & size) == 0;
+                const u64 kx = key[x], ky = key[y];
+                if ((kx > ky) == up) {
+                    const u32 v = val[x];
+                    key[x] = ky;
+                    key[y] = kx;
+                    val[x] = val[y];
+                    val[y] = v;
+                }
+            }
+            __syncthreads();
+        }
+    u32 carry = 0;
+    for (int base = 0; base < n; base += ACC_T) {
+        const int i = base + t;
+        u32 c = 0, nf = 0;
+        if (i < n) {
+            c = val[i];
+            nf = w.c_nfree[c];
+            o.acc[i] = (int)c;
+            o.trk_view[i] = b.V > 1 ? (int)(key[i] >> kb) : 0;
+        }
+        u32 incl = nf;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const u32 x = __shfl_up_sync(0xffffffffu, incl, s);
+            if (lane >= s) incl += x;
+        }
+        if (lane == 31) wsum[wib] = incl;
+        __syncthreads();
+        u32 ws = wsum[lane];   // every warp scans the warp sums
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const u32 x = __shfl_up_sync(0xffffffffu, ws, s);
+            if (lane >= s) ws += x;
+        }
+        const u32 before = wib ? __shfl_sync(0xffffffffu, ws, wib - 1) : 0u;
+        if (i < n) o.trk_moff[i] = (u64)(carry + before + incl - nf);
+        carry += __shfl_sync(0xffffffffu, ws, 31);
+        __syncthreads();
+    }
+    if (t == 0) {
+        o.trk_moff[n] = carry;
+        b.ctl->n_out_members = carry;
+    }
+    for (int v = t; v <= b.V; v += ACC_T) {   // first track of view v
+        int lo = 0, hi = n;
+        if (b.V == 1) lo = v ? n : 0;
+        else
+            while (lo < hi) {
+                const int mid = (lo + hi) / 2;
+                if ((long long)(key[mid] >> kb) < v) lo = mid + 1;
+                else hi = mid;
+            }
+        o.view_trk[v] = lo;
     }
 }
 
@@ -610,6 +709,8 @@ int bits_for(unsigned long long maxval) {
 
 int merge_grid_blocks(int device) {
     cudaFuncSetAttribute(k_long_members, cudaFuncAttributeMaxDynamicSharedMemorySize, LONG_BITS / 8);
+    cudaFuncSetAttribute(k_acc_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(ACC_SMALL * (sizeof(u64) + sizeof(u32))));
     int sms = 0, per_sm = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_merge, MT, 0);
@@ -638,19 +739,30 @@ void launch_single_pass(const Batch &b, const Work &w, cudaStream_t st) {
     launch_dep(k_sp_own, dim3(g), dim3(256), 0, st, b, w);
 }
 
+static void launch_fit(const Batch &b, const Work &w, const Out &o, cudaStream_t st) {
+    launch_dep(k_fit, dim3(sm_count() * 4), dim3(FIT_T), 0, st, b, w, o);
+    launch_dep(k_long_members, dim3(std::min(16u, sm_count())), dim3(LONG_T), (size_t)(LONG_BITS / 8), st, b, w, o);
+}
+
 // Accepted list sorted by (view, key); per-view track offsets; member offsets;
 // fit with the sorted members.  acc_cap sizes the launches; the device counters
 // decide the work.
 void launch_output(const Batch &b, const Work &w, Out &o, long long acc_cap, void *temp, cudaStream_t st) {
     const unsigned g = sm_count() * 4;
-    launch_dep(k_collect, dim3(g), dim3(256), 0, st, b, w, o);
+    const int vbits = bits_for((unsigned long long)std::max(b.V - 1, 0));
+    if (b.N / b.H <= ACC_SMALL && 3 * b.rbits + vbits < 64) {   // a track owns at least H grains
+        launch_dep(k_acc_small, dim3(1), dim3(ACC_T), ACC_SMALL * (sizeof(u64) + sizeof(u32)), st, b, w, o);
+        launch_fit(b, w, o, st);
+        return;
+    }
+    launch_dep(k_acc_keys, dim3(g), dim3(256), 0, st, b, w, o);
     u64 *na = &b.ctl->n_acc;
     int cur = radix_sort_pairs_dev(o.sort_k[0], o.sort_v[0], o.sort_k[1], o.sort_v[1], acc_cap, na, 3 * b.rbits,
                                    temp, st, &b.ctl->error, ERRB_TIMEOUT, b.ctl->bar, b.spin_limit);
     if (b.V > 1) {
         launch_dep(k_view_keys, dim3(g), dim3(256), 0, st, b, w, o.sort_k[cur], o.sort_v[cur]);
         int c2 = radix_sort_pairs_dev(o.sort_k[cur], o.sort_v[cur], o.sort_k[cur ^ 1], o.sort_v[cur ^ 1], acc_cap,
-                                      na, bits_for((unsigned long long)(b.V - 1)), temp, st, &b.ctl->error, ERRB_TIMEOUT,
+                                      na, vbits, temp, st, &b.ctl->error, ERRB_TIMEOUT,
                                       b.ctl->bar, b.spin_limit);
         cur = c2 ? (cur ^ 1) : cur;
     }
@@ -661,8 +773,7 @@ void launch_output(const Batch &b, const Work &w, Out &o, long long acc_cap, voi
                                &b.ctl->error, ERRB_TIMEOUT, b.ctl->bar, b.spin_limit);
     exclusive_scan_u64_dev(o.trk_moff, o.trk_moff, acc_cap, na, temp, &b.ctl->n_out_members, st, &b.ctl->error,
                            ERRB_TIMEOUT, b.ctl->bar, b.spin_limit);
-    launch_dep(k_fit, dim3(g), dim3(FIT_T), 0, st, b, w, o);
-    launch_dep(k_long_members, dim3(std::min(16u, sm_count())), dim3(LONG_T), (size_t)(LONG_BITS / 8), st, b, w, o);
+    launch_fit(b, w, o, st);
 }
 
 }  // namespace et

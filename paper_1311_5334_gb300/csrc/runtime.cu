@@ -618,6 +618,7 @@ Work BatchRT::dev_work() const {
     w.c_moff = c_moff;
     w.c_state = c_state;
     w.c_nfree = c_nfree;
+    w.acc = trk_view;   // the tracks' views are written from the sorted list only
     w.cand_cap = cap_cand;
     w.members = members;
     w.member_cap = cap_members;
