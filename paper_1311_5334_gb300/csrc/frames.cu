@@ -2,32 +2,34 @@
 // camera frames (Section 2 of the paper, Fig. 2), from a batch of views to
 // their grains, and the C ABI of include/et_frames.h.
 //
-// One kernel does both steps.  A block owns a tile of TX x TY pixels of one
-// view and walks its frames front to back.  The frames reach shared memory
-// by TMA (a 3D tensor map over the raw bytes, one box of TX x (TY + 2)
-// pixels per frame: the tile plus one halo row above and below), through a
-// ring of NSTAGE buffers with one mbarrier each.  The block's warps then run
-// independently: each scans its four rows of the tile and, once done with
-// a frame, counts itself out of that frame's stage; the last warp to let go
-// of a stage loads the frame NSTAGE further on into it.  No block-wide
-// barrier is taken inside the frame loop.
+// One kernel does both steps, k_recognize.  Filtering is monotone in the raw
+// value (non-increasing), so f > T holds exactly for raw values below a
+// per-pixel cutoff: the count of raw values whose filtered value exceeds T,
+// computed once per calibration by k_cutoff from the same formula.  A block
+// owns a tile of pixels (256 x 16 on wide frames) and ZC frames: a thread keeps
+// the cutoffs of 16 pixels in registers and compares them with its ZC x 16 raw
+// bytes, four bytes at a time (SWAR), all loads issued before the first is
+// used.  The few voxels that pass (0.2 % of an emulsion view) go to a queue in
+// shared memory; once the tile is scanned the block's warps take them 32 at a
+// time, one per lane: the lane filters the 3 x 3 x 3 box (its own frame first;
+// most candidates end there), applies the maximum test with the raster-order
+// tie rule and computes the exact centre-of-mass sums.  The box's bytes were
+// loaded by this block or its neighbours a moment ago, so they come from the
+// caches.
 //
-// Filtering is monotone in the raw value (non-increasing), so f > T holds
-// exactly for raw values below a per-pixel cutoff: the count of raw values
-// whose filtered value exceeds T, computed once per calibration by
-// k_cutoff from the same formula.  The scan of a frame therefore compares 16
-// raw bytes per lane against 16 cutoffs held in registers (four byte-wise
-// SIMD compares).  The warp then evaluates its rare candidates one at a time
-// with one neighbour of the 3 x 3 x 3 box per lane (halo columns outside the
-// tile come from global memory): one ballot decides the maximum test with the
-// raster-order tie rule (lanes are in raster order, the candidate is lane 13),
-// warp reductions give the exact centre-of-mass sums.  A grain is appended
-// with its key (view, frame, row, column); a radix sort by key then gives
-// every view's grains in raster order, independent of the order blocks ran in.
-#include <cuda.h>
-
+// A grain is counted in its image row (view, frame, row) and linked to the
+// row's grains found before it.  The scan of the row counts gives every row's
+// place in raster order (and the views' offsets), and k_fr_place ranks each
+// grain among its row's few by x.  So the order is independent of the order
+// blocks ran in, without a sort.
+//
+// An earlier form walked each tile's frames through a TMA ring and evaluated
+// candidates one at a time with a neighbour per lane: 0.64 ms for 24 full
+// views, bound by instruction issue at 0.3 of the copy bandwidth; pruning the
+// candidates inside the scanning threads instead took 0.58 ms for the scan
+// alone, the lanes of a warp idling while a few of them prune.
+#include <algorithm>
 #include <cstring>
-#include <mutex>
 
 #include "et_frames.h"
 #include "runtime.h"
@@ -36,18 +38,9 @@ namespace et {
 
 namespace {
 
-constexpr int TX = 256, TY = 16, FT = 256;
-constexpr int LPR = TX / 16;              // lanes per tile row (16 pixels each)
-constexpr int RPW = 32 / LPR;             // tile rows per warp
-constexpr int NSTAGE = 6;
-constexpr int STAGE_BYTES = TX * (TY + 2);
-// calibration tile: the pixel tile with one halo row above and below and 16
-// columns on either side (so that it loads as aligned 16-byte vectors); pixel
-// column lx of the tile is calibration column lx + 16
-constexpr int HX = TX + 32, HY = TY + 2;
-static_assert(FT == LPR * TY, "one thread per 16 pixels of the tile");
-static_assert(STAGE_BYTES % 128 == 0, "stage buffers stay 128-byte aligned");
-static_assert(TX <= 256 && TY + 2 <= 256, "TMA box edges are at most 256 elements");
+constexpr int FT = 256;       // threads per block
+constexpr int ZC = 8;         // frames a scanning thread holds at a time
+constexpr int QCAP = 16 * FT; // candidates a block collects on chip: at least one frame of its tile
 
 enum : u32 { FRB_OVF = 1u << 0, FRB_TIMEOUT = 1u << 1 };
 
@@ -55,7 +48,7 @@ struct FrCtl {
     u64 n_grains;   // grains appended (may exceed the capacity)
     u64 n_cand;     // voxels with f > T
     u32 error;      // FRB_* bits
-    u32 bar[2];     // grid barrier of the sort and the scan
+    u32 bar[2];     // grid barrier of the scan
     u32 pad;
 };
 
@@ -63,16 +56,20 @@ struct FrArgs {
     int W, H, D, P, V;
     int T;
     int num[3], den[3];
-    int tiles_x;
-    const unsigned char *raw;   // device copy of the views (halo columns of candidates)
+    int chunks;                 // 16-pixel chunks per row
+    int zb;                     // frames of a block, a multiple of ZC
+    int lc, tiles_x;            // a tile is 2^lc chunks wide and FT / 2^lc rows high; tiles per row
+    const unsigned char *raw;
     const unsigned char *gain, *thr, *cut;   // padded tables: pixel (x, y) at (y + 1) * TP + x + 16
+    const unsigned short *cal;               // gain | thr << 8, same layout
     int TP;
     FrCtl *ctl;
-    u64 *keys;
-    u32 *vals;
+    u64 *key;                   // row << 12 | x
+    u32 *next;                  // grain of the same row found before (~0: none)
     int4 *rec;
     u64 cap;
-    u32 *view_count;
+    u32 *row_count;             // per image row: grains, then (row_head) the last one found
+    u32 *row_head;
 };
 
 __device__ __forceinline__ int filt(int raw, int g, int t) {
@@ -82,322 +79,217 @@ __device__ __forceinline__ int filt(int raw, int g, int t) {
 
 // Per pixel: the number of raw values r in [0, 255] with filt(r) > T; by
 // monotonicity exactly the r below it.  filt(255) = 0, so it is at most 255.
-__global__ void k_cutoff(const unsigned char *gain, const unsigned char *thr, unsigned char *cut, int n, int T) {
+__global__ void k_cutoff(const unsigned char *gain, const unsigned char *thr, unsigned char *cut, unsigned short *cal,
+                         int n, int T) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int g = gain[i], t = thr[i];
         int c = 0;
         for (int r = 0; r < 256; ++r) c += filt(r, g, t) > T;
         cut[i] = (unsigned char)c;
+        cal[i] = (unsigned short)(g | (t << 8));
     }
 }
 
-__device__ __forceinline__ u32 smem_addr(const void *p) { return (u32)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ u64 global_ns() {
-    u64 t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Waits for the phase `parity` of the mbarrier at bar; false after about a
-// second without completion (the caller records a timeout and leaves).
-__device__ __forceinline__ bool mbar_try(u32 bar, u32 parity) {
-    u32 done;
-    // suspends for up to 2 us while the phase is pending instead of spinning
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity), "r"(2000)
-        : "memory");
-    return done != 0;
-}
-
-__device__ __noinline__ bool mbar_wait_slow(u32 bar, u32 parity) {
-    const u64 t0 = global_ns();
-    for (u32 it = 0;; ++it) {
-        if (mbar_try(bar, parity)) return true;
-        if ((it & 7) == 7 && global_ns() - t0 > 1000000000ull) return false;
-        if (it > (1u << 26)) return false;
-    }
-}
-
-// Waits for the phase `parity` of the mbarrier at bar; false after about a
-// second without completion (the caller records a timeout and leaves).
-__device__ __forceinline__ bool mbar_wait(u32 bar, u32 parity) {
-    return mbar_try(bar, parity) || mbar_wait_slow(bar, parity);
-}
-
-__global__ void __launch_bounds__(FT, 5) k_recognize(const __grid_constant__ CUtensorMap tmap, FrArgs a) {
-    __shared__ __align__(128) unsigned char stage[NSTAGE][STAGE_BYTES];
-    __shared__ __align__(16) unsigned char gsm[HY][HX];
-    __shared__ __align__(16) unsigned char tsm[HY][HX];
-    __shared__ __align__(8) u64 mbar[NSTAGE];
-    __shared__ int released[NSTAGE];   // warps done with the frame a stage holds
-    __shared__ int issued;             // frames whose load has been issued
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int v = blockIdx.y;
-    const int x0 = (blockIdx.x % a.tiles_x) * TX, y0 = (blockIdx.x / a.tiles_x) * TY;
-    const int D = a.D;
-
-    auto issue = [&](int j, int s) {   // TMA of frame j of this view into stage s = j % NSTAGE
-        const u32 bar = smem_addr(&mbar[s]);
-        // the stage was last read by ordinary loads of every warp (released below)
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(STAGE_BYTES)
-                     : "memory");
-        asm volatile(
-            "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-            "[%5];" ::"r"(smem_addr(stage[s])),
-            "l"(&tmap), "r"(x0), "r"(y0 - 1), "r"(v * D + j), "r"(bar)
-            : "memory");
-    };
-
-    if (tid == 0) {
-        for (int s = 0; s < NSTAGE; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbar[s])) : "memory");
-            released[s] = 0;
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        issued = min(D, NSTAGE);
-    }
-    __syncthreads();
-    if (tid == 0)
-        for (int j = 0; j < min(D, NSTAGE); ++j) issue(j, j);
-
-    // calibration of the tile with its halo and margins (zero outside the frame)
-    for (int i = tid; i < HY * (HX / 16); i += FT) {
-        const int row = i / (HX / 16), c16 = (i % (HX / 16)) * 16;
-        const size_t off = (size_t)(y0 + row) * a.TP + x0 + c16;
-        *(uint4 *)&gsm[row][c16] = __ldg((const uint4 *)(a.gain + off));
-        *(uint4 *)&tsm[row][c16] = __ldg((const uint4 *)(a.thr + off));
-    }
-    // this lane's 16 pixels: row ry of the tile (warp w scans rows RPW w ..
-    // RPW w + RPW - 1), columns cx .. cx + 15, and their cutoffs
-    const int ry = tid / LPR, cx = (tid % LPR) * 16;
-    u32 cw[4];   // cutoffs of the 16 pixels, 4 per word, low 7 bits of each byte
-    u32 ch[4];   // and their high bits
-    {
-        const uint4 c = __ldg((const uint4 *)(a.cut + (size_t)(y0 + ry + 1) * a.TP + x0 + cx + 16));
-        const u32 cv[4] = {c.x, c.y, c.z, c.w};
+// Tests the candidate (x, y, z) of view v and appends its grain if it is a
+// maximum of its 3 x 3 x 3 box.
+__device__ __noinline__ void test_candidate(const FrArgs &a, int x, int y, int z, int v) {
+    const size_t frame = (size_t)a.H * a.P;
+    const unsigned char *at = a.raw + ((size_t)v * a.D + z) * frame + (size_t)y * a.P;   // row start
+    const unsigned short *cal = a.cal + (size_t)(y + 1) * a.TP + x + 16;
+    u32 c[9];   // calibration of the 3 x 3 pixels
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            cw[k] = cv[k] & 0x7f7f7f7fu;
-            ch[k] = cv[k] & 0x80808080u;
+    for (int k = 0; k < 9; ++k) c[k] = __ldg(cal + (k / 3 - 1) * a.TP + k % 3 - 1);
+    // raw bytes x - 1, x, x + 1 of a row in the low 24 bits
+    const int xs = max(x - 1, 0), xw = xs & ~3, sh = 8 * (xs & 3);
+    const bool two = (xs & 3) >= 2 && xw + 4 < a.P;
+    auto row3 = [&](const unsigned char *row) {
+        const u32 w0 = __ldg((const u32 *)(row + xw));
+        const u32 w1 = two ? __ldg((const u32 *)(row + xw + 4)) : 0u;
+        const u32 w = __funnelshift_r(w0, w1, sh);
+        return x > 0 ? w : w << 8;
+    };
+    const bool left = x > 0, right = x + 1 < a.W;
+    auto value = [&](u32 w, int dy, int k) {   // filtered value of byte k (dx = k - 1); outside the frame: -1
+        if ((k == 0 && !left) || (k == 2 && !right)) return -1;
+        const u32 cc = c[(dy + 1) * 3 + k];
+        return filt((int)(w >> (8 * k)) & 255, (int)(cc & 255u), (int)(cc >> 8));
+    };
+    int S = 0, SX = 0, SY = 0, SZ = 0;
+    auto sum = [&](int f, int dx, int dy, int dz) {
+        f = max(f, 0);
+        S += f;
+        SX += dx * f;
+        SY += dy * f;
+        SZ += dz * f;
+    };
+    bool alive = true;
+    u32 w[3];   // the candidate's frame
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy)
+        w[dy + 1] = (unsigned)(y + dy) < (unsigned)a.H ? row3(at + (ptrdiff_t)dy * a.P) : 0u;
+    const int fc = value(w[1], 0, 1);
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy) {
+        if ((unsigned)(y + dy) >= (unsigned)a.H) continue;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int f = value(w[dy + 1], dy, k);
+            const bool before = dy < 0 || (dy == 0 && k == 0);
+            if (dy != 0 || k != 1) alive = alive && (before ? f < fc : f <= fc);
+            sum(f, k - 1, dy, 0);
         }
     }
-    __syncthreads();   // calibration tiles complete; from here on the warps run independently
-
-    // this lane's neighbour in a candidate's 3 x 3 x 3 box (lanes 0..26, raster
-    // order, so lane 13 is the candidate and lanes below it come before it)
-    const int ndz = lane / 9 - 1, ndy = (lane / 3) % 3 - 1, ndx = lane % 3 - 1;
-    // the centroid coordinate this lane computes for a grain (lanes 0, 1, 2)
-    const int cnum = lane == 0 ? a.num[0] : (lane == 1 ? a.num[1] : a.num[2]);
-    const int cden = lane == 0 ? a.den[0] : (lane == 1 ? a.den[1] : a.den[2]);
-    u32 ncand = 0;
-    u32 fprev[4] = {0u, 0u, 0u, 0u};
-    bool timed_out = false;
-    // stages of frames z - 1, z, z + 1 and the phase parity of frame z + 1
-    int sm1 = NSTAGE - 1, s0 = 0, sp1 = 1;
-    u32 par1 = 0;
-    if (!mbar_wait(smem_addr(&mbar[0]), 0)) timed_out = true;
-    for (int z = 0; z < D && !timed_out; ++z) {
-        if (z + 1 < D && !mbar_wait(smem_addr(&mbar[sp1]), par1)) {
-            timed_out = true;
-            break;
+    if (!alive) return;
+#pragma unroll
+    for (int dz = -1; dz <= 1; dz += 2) {   // the frames before and after
+        if ((unsigned)(z + dz) >= (unsigned)a.D) continue;
+        const unsigned char *fr = at + (ptrdiff_t)dz * (ptrdiff_t)frame;
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy)
+            w[dy + 1] = (unsigned)(y + dy) < (unsigned)a.H ? row3(fr + (ptrdiff_t)dy * a.P) : 0u;
+#pragma unroll
+        for (int dy = -1; dy <= 1; ++dy) {
+            if ((unsigned)(y + dy) >= (unsigned)a.H) continue;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int f = value(w[dy + 1], dy, k);
+                alive = alive && (dz < 0 ? f < fc : f <= fc);
+                sum(f, k - 1, dy, dz);
+            }
         }
-        // scan: this lane's pixels of frame z whose raw value is below the cutoff
-        const unsigned char *f0 = stage[s0];
-        const uint4 rw = *(const uint4 *)&f0[(ry + 1) * TX + cx];
+    }
+    if (!alive) return;
+    const unsigned won = __activemask();   // the lanes here together share one atomic
+    const int lane = threadIdx.x & 31, leader = __ffs(won) - 1;
+    u64 slot = 0;
+    if (lane == leader) slot = atomicAdd(&a.ctl->n_grains, (u64)__popc(won));
+    slot = __shfl_sync(won, slot, leader) + __popc(won & ((1u << lane) - 1u));
+    if (slot >= a.cap) {
+        atomicOr(&a.ctl->error, FRB_OVF);
+        return;
+    }
+    // coordinate of an axis, rounded half up: floor((2 S g num + 2 So num + S
+    // den) / (2 S den)) with the voxel index g and So the offset sum.  With A =
+    // 2 g num = a1 (2 den) + a0 it is a1 + floor((S a0 + 2 So num + S den) / (2 S
+    // den)), all in int32: A < 2^30, S a0 < 9.1e8, |2 So num| < 3.1e8, S den < 4.6e8
+    auto coord = [&](int g, int So, int axis) {
+        const int A = 2 * g * a.num[axis], twoden = 2 * a.den[axis];
+        const int a1 = A / twoden, a0 = A - a1 * twoden;
+        const int m = S * a0 + 2 * So * a.num[axis] + S * a.den[axis], Q = S * twoden;
+        int q = m / Q;
+        if (m < 0 && q * Q != m) --q;
+        return a1 + q;
+    };
+    const u64 row = ((u64)v * a.D + z) * a.H + y;
+    a.key[slot] = (row << 12) | (u64)x;
+    a.rec[slot] = make_int4(coord(x, SX, 0), coord(y, SY, 1), coord(z, SZ, 2), S);
+    atomicAdd(&a.row_count[row], 1u);
+    a.next[slot] = atomicExch(&a.row_head[row], (u32)slot);
+}
+
+// Tile blockIdx.x of frames blockIdx.y zb .. of view blockIdx.z.  The floor is
+// one read of the raw frames (DRAM).  With many views a block takes the whole
+// depth, whose some 330 candidates keep all its warps busy in the test; with
+// few views the depth is split so that the blocks fill the device.
+__global__ void __launch_bounds__(FT, 4) k_recognize(const __grid_constant__ FrArgs a) {
+    griddep_launch();
+    griddep_wait();
+    __shared__ u32 queue[QCAP];   // thread | pixel << 8 | frame << 12
+    __shared__ u32 queued;
+    static_assert(FT == 256, "bits of a queue entry");
+    const int tid = threadIdx.x;
+    if (tid == 0) queued = 0;
+    __syncthreads();
+    const int tx0 = (blockIdx.x % a.tiles_x) << a.lc, ty0 = (blockIdx.x / a.tiles_x) * (FT >> a.lc);
+    const int chunk = tx0 + (tid & ((1 << a.lc) - 1)), y = ty0 + (tid >> a.lc);
+    const int v = blockIdx.z, z0 = blockIdx.y * a.zb, nz = min(a.zb, a.D - z0);
+    const size_t frame = (size_t)a.H * a.P;
+    const bool mine = chunk < a.chunks && y < a.H;
+    const unsigned char *src = a.raw + ((size_t)v * a.D + z0) * frame + (size_t)y * a.P + chunk * 16;
+    u32 cv[4] = {0u, 0u, 0u, 0u};
+    // queues the pixels of frame kz below their cutoffs
+    auto scan = [&](uint4 r, int kz) {
         // per byte raw < cutoff, four bytes a word (SWAR): with the byte's high
         // bits ra, ca and d = (raw | 0x80) - (cutoff & 0x7f) (no borrow between
         // bytes), raw < cutoff iff (!ra & ca) | (ra == ca & !d7)
-        const u32 rwv[4] = {rw.x, rw.y, rw.z, rw.w};
+        const u32 rw[4] = {r.x, r.y, r.z, r.w};
         u32 lt[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const u32 d = (rwv[k] | 0x80808080u) - cw[k];
-            lt[k] = ((~rwv[k] & ch[k]) | (~(rwv[k] ^ ch[k]) & ~d)) & 0x80808080u;
+            const u32 d = (rw[k] | 0x80808080u) - (cv[k] & 0x7f7f7f7fu);
+            lt[k] = ((~rw[k] & cv[k]) | (~(rw[k] ^ cv[k]) & ~d)) & 0x80808080u;
         }
-        u32 bits = 0;   // bit k: pixel cx + k
         if (lt[0] | lt[1] | lt[2] | lt[3]) {
+            u32 m = (lt[0] >> 7) | (lt[1] >> 6) | (lt[2] >> 5) | (lt[3] >> 4);   // bit 8 j + k: byte j of word k
+            u32 s = atomicAdd(&queued, (u32)__popc(m));
+            for (; m && s < QCAP; m &= m - 1, ++s) {
+                const int bit = __ffs(m) - 1, px = 4 * (bit & 7) + (bit >> 3);
+                queue[s] = (u32)(tid | (px << 8) | (kz << 12));
+            }
+        }
+    };
+    auto test_queue = [&](u32 n) {
+        for (u32 i = tid; i < n; i += FT) {
+            const u32 e = queue[i];
+            const int t = (int)(e & 255u);
+            test_candidate(a, (tx0 + (t & ((1 << a.lc) - 1))) * 16 + (int)((e >> 8) & 15u), ty0 + (t >> a.lc),
+                           z0 + (int)(e >> 12), v);
+        }
+    };
+    if (mine) {
+        const uint4 c4 = __ldg((const uint4 *)(a.cut + (size_t)(y + 1) * a.TP + chunk * 16 + 16));
+        cv[0] = c4.x;
+        cv[1] = c4.y;
+        cv[2] = c4.z;
+        cv[3] = c4.w;
+        for (int z = 0; z < nz; z += ZC) {
+            uint4 r[ZC];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const u32 m = lt[k] >> 7;   // bits 0, 8, 16, 24
-                bits |= ((m & 1u) | ((m >> 7) & 2u) | ((m >> 14) & 4u) | ((m >> 21) & 8u)) << (4 * k);
-            }
-        }
-        // exact pruning inside the lane, before the warp-wide test: filtered
-        // values of the lane's candidates (only candidates can beat a
-        // candidate: every other voxel has f <= T).  Of two candidates next to
-        // each other in x, the earlier loses iff the later is brighter, else
-        // the later loses; a candidate loses to the same pixel one frame back
-        // if that was at least as bright.  fprev: this lane's filtered values
-        // of frame z - 1 (candidates only, else 0), a byte per pixel.
-        u32 fnow[4] = {0u, 0u, 0u, 0u};
-        if (bits) {
-            ncand += __popc(bits);
-            u32 keep = bits, b = bits;
-            int pk = -2, pf = 0;
-            while (b) {
-                const int k = __ffs(b) - 1;
-                b &= b - 1;
-                const int wsel = k >> 2, sh = 8 * (k & 3);
-                const u32 word = wsel == 0 ? rwv[0] : (wsel == 1 ? rwv[1] : (wsel == 2 ? rwv[2] : rwv[3]));
-                const u32 prev = wsel == 0 ? fprev[0] : (wsel == 1 ? fprev[1] : (wsel == 2 ? fprev[2] : fprev[3]));
-                const int f = filt((word >> sh) & 0xffu, gsm[ry + 1][cx + k + 16], tsm[ry + 1][cx + k + 16]);
-                if ((int)((prev >> sh) & 0xffu) >= f) keep &= ~(1u << k);
-                if (pk == k - 1) {
-                    if (pf >= f) keep &= ~(1u << k);
-                    else keep &= ~(1u << pk);
-                }
-                pk = k;
-                pf = f;
-                const u32 ins = (u32)f << sh;
-                fnow[0] |= wsel == 0 ? ins : 0u;
-                fnow[1] |= wsel == 1 ? ins : 0u;
-                fnow[2] |= wsel == 2 ? ins : 0u;
-                fnow[3] |= wsel == 3 ? ins : 0u;
-            }
-            bits = keep;
-        }
+            for (int k = 0; k < ZC; ++k)
+                if (z + k < nz) r[k] = __ldg((const uint4 *)(src + (size_t)(z + k) * frame));
 #pragma unroll
-        for (int k = 0; k < 4; ++k) fprev[k] = fnow[k];
-        unsigned pend = __ballot_sync(0xffffffffu, bits != 0);
-        if (pend) {
-            // per frame: this lane's neighbour (frame, and offsets in the stage and
-            // calibration tiles) and whether its frame exists
-            const int zz = z + ndz;
-            const bool zin = lane < 27 && zz >= 0 && zz < D;
-            const unsigned char *fr = stage[ndz < 0 ? sm1 : (ndz == 0 ? s0 : sp1)] + ndy * TX + ndx;
-            // the warp evaluates its candidates one at a time, a neighbour per lane
-            for (; pend; pend = __ballot_sync(0xffffffffu, bits != 0)) {
-                const int src = __ffs(pend) - 1;
-                const int k = __ffs(__shfl_sync(0xffffffffu, bits, src)) - 1;
-                if (lane == src) bits &= bits - 1;
-                const int lx = (src % LPR) * 16 + k, ly = warp * RPW + src / LPR;   // uniform
-                const int gx = x0 + lx, gy = y0 + ly;
-                const bool in = zin && (unsigned)(gy + ndy) < (unsigned)a.H && (unsigned)(gx + ndx) < (unsigned)a.W;
-                const int sb = (ly + 1) * TX + lx;
-                int r = 0;
-                if (lx > 0 && lx < TX - 1) {   // uniform: the whole box is in the stage
-                    if (in) r = fr[sb];
-                } else if (in) {               // tile edge: halo columns from global memory
-                    r = ((unsigned)(lx + ndx) < (unsigned)TX)
-                            ? fr[sb]
-                            : __ldg(&a.raw[(((size_t)v * D + zz) * a.H + gy + ndy) * (size_t)a.P + gx + ndx]);
-                }
-                const int cb = (ly + 1 + ndy) * HX + lx + ndx + 16;
-                const int fq = in ? filt(r, (&gsm[0][0])[cb], (&tsm[0][0])[cb]) : -1;
-                const int fpv = __shfl_sync(0xffffffffu, fq, 13);
-                const bool beats = lane < 13 ? fq >= fpv : fq > fpv;
-                if (__ballot_sync(0xffffffffu, beats)) continue;   // not a local maximum
-                // centre-of-mass sums, two per reduction: S (< 2^13) below
-                // Sx = sum w dx above; Sy + 4096 (sum of w dy + 128 over 32 lanes, in
-                // [1801, 6391]) below Sz = sum w dz above
-                const int w = max(fq, 0);
-                const int p1 = __reduce_add_sync(0xffffffffu, (u32)(w + ndx * w * 65536));
-                const int p2 = __reduce_add_sync(0xffffffffu, (u32)(ndy * w + 128 + ndz * w * 65536));
-                const int S = p1 & 0xffff, SXo = (p1 - S) >> 16;
-                const int SYo = (p2 & 0xffff) - 4096, SZo = (p2 - (p2 & 0xffff)) >> 16;
-                // coordinate of axis `lane` (lanes 0..2), rounded half up:
-                // floor((2 S g num + 2 So num + S den) / (2 S den)) with the voxel
-                // index g and So the offset sum.  With A = 2 g num = a1 (2 den) + a0
-                // it is a1 + floor((S a0 + 2 So num + S den) / (2 S den)), all in
-                // int32: A < 2^30, S a0 < 9.1e8, |2 So num| < 3.1e8, S den < 4.6e8
-                int c = 0;
-                if (lane < 3) {
-                    const int g = lane == 0 ? gx : (lane == 1 ? gy : z);
-                    const int So = lane == 0 ? SXo : (lane == 1 ? SYo : SZo);
-                    const int A = 2 * g * cnum, twoden = 2 * cden;
-                    const int a1 = A / twoden, a0 = A - a1 * twoden;
-                    const int n = S * a0 + 2 * So * cnum + S * cden, Q = S * twoden;
-                    int q = n / Q;
-                    if (n < 0 && q * Q != n) --q;
-                    c = a1 + q;
-                }
-                const int Y = __shfl_sync(0xffffffffu, c, 1), Z = __shfl_sync(0xffffffffu, c, 2);
-                if (lane == 0) {
-                    const u64 slot = atomicAdd(&a.ctl->n_grains, 1ull);
-                    if (slot < a.cap) {
-                        a.keys[slot] = (u64)v * ((u64)D * a.H * a.W) + ((u64)z * a.H + gy) * a.W + gx;
-                        a.vals[slot] = (u32)slot;
-                        a.rec[slot] = make_int4(c, Y, Z, S);
-                    } else {
-                        atomicOr(&a.ctl->error, FRB_OVF);
-                    }
-                    atomicAdd(&a.view_count[v], 1u);
-                }
-            }
+            for (int k = 0; k < ZC; ++k)
+                if (z + k < nz) scan(r[k], z + k);
         }
-        // frame z - 1 is no longer needed by this warp; the last warp to let go
-        // of it reloads its stage with frame z + NSTAGE - 1
-        __syncwarp();
-        if (lane == 0 && z >= 1) {
-            __threadfence_block();
-            if (atomicAdd(&released[sm1], 1) == FT / 32 - 1) {
-                released[sm1] = 0;
-                __threadfence_block();
-                const int j = z - 1 + NSTAGE;
-                if (j < D) {
-                    issue(j, sm1);
-                    atomicAdd(&issued, 1);
-                }
-            }
-        }
-        sm1 = s0;
-        s0 = sp1;
-        if (++sp1 == NSTAGE) {
-            sp1 = 0;
-            par1 ^= 1u;
-        }
-    }
-    ncand = __reduce_add_sync(0xffffffffu, ncand);
-    if (lane == 0 && ncand) atomicAdd(&a.ctl->n_cand, (u64)ncand);
-    if (timed_out && lane == 0) {
-        // record the failure; the block's first warp then gives the copies still
-        // in flight into its buffers a bounded chance to land before it exits
-        atomicOr(&a.ctl->error, FRB_TIMEOUT);
     }
     __syncthreads();
-    if (tid == 0 && (*(volatile u32 *)&a.ctl->error & FRB_TIMEOUT)) {
-        const int n = *(volatile int *)&issued;
-        for (int j = max(0, n - NSTAGE); j < n; ++j)
-            if (!mbar_wait(smem_addr(&mbar[j % NSTAGE]), (j / NSTAGE) & 1)) break;
+    const u32 all = queued;
+    if (tid == 0 && all) atomicAdd(&a.ctl->n_cand, (u64)all);
+    if (all <= QCAP) {
+        test_queue(all);
+        return;
+    }
+    // a crowded tile: again, a frame at a time (its candidates always fit)
+    for (int k = 0; k < nz; ++k) {
+        __syncthreads();
+        if (tid == 0) queued = 0;
+        __syncthreads();
+        if (mine) scan(__ldg((const uint4 *)(src + (size_t)k * frame)), k);
+        __syncthreads();
+        test_queue(queued);
     }
 }
 
-// Grains in key order: xyz (int32 [n][3]) and pulse (int32 [n]).
-__global__ void k_fr_gather(const FrCtl *ctl, u64 cap, const u32 *sorted_vals, const int4 *rec, int *xyz,
-                            int *pulse) {
-    const u64 n = min(ctl->n_grains, cap);
-    for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
-        const int4 r = rec[sorted_vals[i]];
-        xyz[3 * i + 0] = r.x;
-        xyz[3 * i + 1] = r.y;
-        xyz[3 * i + 2] = r.z;
-        pulse[i] = r.w;
+// Grains into raster order: a grain's place is its row's start plus its rank by
+// x among the row's grains (a few).  Also the views' offsets.
+__global__ void k_fr_place(FrArgs a, const u32 *row_start, int *xyz, int *pulse, u32 *view_off) {
+    griddep_launch();
+    griddep_wait();
+    const u64 n = min(a.ctl->n_grains, a.cap);
+    const u64 tid = (u64)blockIdx.x * blockDim.x + threadIdx.x, stride = (u64)gridDim.x * blockDim.x;
+    for (u64 v = tid; v <= (u64)a.V; v += stride) view_off[v] = row_start[v * (u64)a.D * a.H];
+    for (u64 i = tid; i < n; i += stride) {
+        const u64 k = a.key[i], row = k >> 12;
+        u32 rank = 0;
+        for (u32 j = a.row_head[row]; j != ~0u; j = a.next[j]) rank += a.key[j] < k;
+        const u64 p = (u64)row_start[row] + rank;
+        if (p >= a.cap) continue;   // only after an overflow, when the run is repeated
+        const int4 r = a.rec[i];
+        xyz[3 * p + 0] = r.x;
+        xyz[3 * p + 1] = r.y;
+        xyz[3 * p + 2] = r.z;
+        pulse[p] = r.w;
     }
-}
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)p;
-    });
-    return fn;
 }
 
 }  // namespace
@@ -408,18 +300,19 @@ struct FramesRT {
     et_frame_params p;
     Group g_tab, g_raw, g_out, g_ctl;
     unsigned char *gain = nullptr, *thr = nullptr, *cut = nullptr;
+    unsigned short *cal = nullptr;
     FrCtl *ctl = nullptr;
     // run state
     int V = 0;
     const unsigned char *d_raw = nullptr;
     u64 cap = 0, want = 0;
-    u64 *keys[2] = {nullptr, nullptr};
-    u32 *vals[2] = {nullptr, nullptr};
+    u64 *key = nullptr;
+    u32 *next = nullptr;
     int4 *rec = nullptr;
     int *xyz = nullptr, *pulse = nullptr;
-    u32 *view_count = nullptr, *view_off = nullptr;
+    u32 *row_count = nullptr, *row_head = nullptr, *row_start = nullptr, *view_off = nullptr;
     void *temp = nullptr;
-    int sorted = 0, launches = 0;
+    int launches = 0;
     cudaStream_t run_stream = nullptr;
     cudaEvent_t ev[4] = {};   // run start, kernel start, kernel end, done
     cudaEvent_t handoff = nullptr;   // a batch's copy of the grains (et_frames_to_batch)
@@ -443,12 +336,11 @@ struct FramesRT {
     }
 
     size_t pixels() const { return (size_t)p.width * p.height; }
-    // padded calibration tables: pitch covering every tile plus 16-byte margins,
-    // one row above and enough below for the last tile's halo
-    int tiles_x() const { return (p.width + TX - 1) / TX; }
-    int tiles_y() const { return (p.height + TY - 1) / TY; }
-    int table_pitch() const { return tiles_x() * TX + 32; }
-    size_t table_bytes() const { return (size_t)table_pitch() * ((size_t)tiles_y() * TY + 2); }
+    // padded calibration tables: 16 columns on either side (16-byte loads), one row
+    // above and below
+    int table_pitch() const { return (p.width + 15) / 16 * 16 + 32; }
+    size_t table_bytes() const { return (size_t)table_pitch() * ((size_t)p.height + 2); }
+    size_t rows() const { return (size_t)V * p.depth * p.height; }
     size_t view_bytes() const { return (size_t)p.depth * p.height * p.row_pitch; }
 
     et_status init() {
@@ -457,10 +349,11 @@ struct FramesRT {
         if (cudaEventCreateWithFlags(&handoff, cudaEventDisableTiming) != cudaSuccess)
             return fail(ET_ERR_CUDA, "event creation failed");
         const size_t tb = align_up(table_bytes(), 256);
-        if (!g_tab.reserve(ctx, 3 * tb)) return fail(ET_ERR_OOM, "calibration tables");
+        if (!g_tab.reserve(ctx, 5 * tb)) return fail(ET_ERR_OOM, "calibration tables");
         gain = (unsigned char *)g_tab.base;
         thr = gain + tb;
         cut = thr + tb;
+        cal = (unsigned short *)(cut + tb);
         if (!g_ctl.reserve(ctx, sizeof(FrCtl))) return fail(ET_ERR_OOM, "control block");
         ctl = (FrCtl *)g_ctl.base;
         return ET_OK;
@@ -478,7 +371,7 @@ struct FramesRT {
         if (e != cudaSuccess) return cuda_fail(e, "calibration upload");
         // zero gain outside the frame gives a zero cutoff there
         const int n = (int)table_bytes();
-        k_cutoff<<<std::min((n + 255) / 256, 152 * 8), 256, 0, st>>>(gain, thr, cut, n, p.grain_threshold);
+        k_cutoff<<<std::min((n + 255) / 256, 152 * 8), 256, 0, st>>>(gain, thr, cut, cal, n, p.grain_threshold);
         e = cudaStreamSynchronize(st);   // the caller may free its tables on return
         return e == cudaSuccess ? ET_OK : cuda_fail(e, "cutoff table");
     }
@@ -486,16 +379,16 @@ struct FramesRT {
     et_status reserve_out(u64 need) {
         Carver c;
         auto carve = [&](Carver &cv) {
-            keys[0] = cv.take<u64>(need);
-            keys[1] = cv.take<u64>(need);
-            vals[0] = cv.take<u32>(need);
-            vals[1] = cv.take<u32>(need);
+            key = cv.take<u64>(need);
+            next = cv.take<u32>(need);
             rec = cv.take<int4>(need);
             xyz = cv.take<int>(3 * need);
             pulse = cv.take<int>(need);
-            view_count = cv.take<u32>((size_t)V + 1);
+            row_count = cv.take<u32>(rows());
+            row_head = cv.take<u32>(rows());
+            row_start = cv.take<u32>(rows() + 1);
             view_off = cv.take<u32>((size_t)V + 1);
-            temp = cv.take<char>(std::max(radix_temp_bytes((long long)need), scan_temp_bytes((long long)V)));
+            temp = cv.take<char>(scan_temp_bytes((long long)rows()));
         };
         carve(c);
         if (!g_out.reserve(ctx, c.off)) return fail(ET_ERR_OOM, "grain buffers (%llu grains)", (unsigned long long)need);
@@ -503,25 +396,16 @@ struct FramesRT {
         d.base = g_out.base;
         carve(d);
         cap = need;
+        last_views = (size_t)V;   // the views the row arrays are carved for
         return ET_OK;
     }
 
     et_status enqueue(cudaStream_t st) {
-        const int tiles_x = (p.width + TX - 1) / TX, tiles_y = (p.height + TY - 1) / TY;
-        EncodeTiledFn enc = encode_fn();
-        if (!enc) return fail(ET_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-        CUtensorMap tmap;
-        const cuuint64_t dims[3] = {(cuuint64_t)p.width, (cuuint64_t)p.height, (cuuint64_t)V * p.depth};
-        const cuuint64_t strides[2] = {(cuuint64_t)p.row_pitch, (cuuint64_t)p.row_pitch * p.height};
-        const cuuint32_t box[3] = {TX, TY + 2, 1};
-        const cuuint32_t estr[3] = {1, 1, 1};
-        CUresult r = enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, (void *)d_raw, dims, strides, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(ET_ERR_CUDA, "tensor map encoding failed (%d)", (int)r);
         cudaMemsetAsync(ctl, 0, sizeof(FrCtl), st);
-        cudaMemsetAsync(view_count, 0, sizeof(u32) * ((size_t)V + 1), st);
+        cudaMemsetAsync(row_count, 0, sizeof(u32) * rows(), st);
+        cudaMemsetAsync(row_head, 0xFF, sizeof(u32) * rows(), st);
         FrArgs a;
+        memset(&a, 0, sizeof a);
         a.W = p.width;
         a.H = p.height;
         a.D = p.depth;
@@ -532,29 +416,35 @@ struct FramesRT {
             a.num[k] = p.pitch_num[k];
             a.den[k] = p.pitch_den[k];
         }
-        a.tiles_x = tiles_x;
+        a.chunks = (p.width + 15) / 16;
+        while (a.lc < 4 && (1 << a.lc) < a.chunks) ++a.lc;
+        a.tiles_x = (a.chunks + (1 << a.lc) - 1) >> a.lc;
+        const int tile_h = FT >> a.lc, tiles_y = (p.height + tile_h - 1) / tile_h;
         a.raw = d_raw;
         a.gain = gain;
         a.thr = thr;
         a.cut = cut;
+        a.cal = cal;
         a.TP = table_pitch();
         a.ctl = ctl;
-        a.keys = keys[0];
-        a.vals = vals[0];
+        a.key = key;
+        a.next = next;
         a.rec = rec;
         a.cap = cap;
-        a.view_count = view_count;
+        a.row_count = row_count;
+        a.row_head = row_head;
         cudaEventRecord(ev[1], st);
-        k_recognize<<<dim3(tiles_x * tiles_y, V), FT, 0, st>>>(tmap, a);
+        // the depth in as few pieces as give the device 8 blocks per SM
+        const long long tiles = (long long)a.tiles_x * tiles_y * V;
+        const int steps = (p.depth + ZC - 1) / ZC;
+        const int pieces = (int)std::min<long long>(steps, std::max<long long>(1, (152 * 8 + tiles - 1) / tiles));
+        a.zb = (steps + pieces - 1) / pieces * ZC;
+        launch_dep(k_recognize, dim3((unsigned)(a.tiles_x * tiles_y), (unsigned)((p.depth + a.zb - 1) / a.zb), (unsigned)V),
+                   dim3(FT), 0, st, a);
         cudaEventRecord(ev[2], st);
-        const int bits = bits_for((u64)V * p.depth * p.height * p.width - 1);
-        sorted = radix_sort_pairs_dev(keys[0], vals[0], keys[1], vals[1], (long long)cap, &ctl->n_grains, bits,
-                                      temp, st, &ctl->error, FRB_TIMEOUT, ctl->bar);
-        // recognition, the sort, the gather and the scan of the view counts
-        launches = 1 + radix_sort_launches(bits) + 1 + 1;
-        k_fr_gather<<<152 * 4, 256, 0, st>>>(ctl, cap, vals[sorted], rec, xyz, pulse);
-        exclusive_scan_u32(view_count, view_off, (long long)V, temp, st, &ctl->error, FRB_TIMEOUT,
-                           ctl->bar);   // view_off[V] = total
+        exclusive_scan_u32(row_count, row_start, (long long)rows(), temp, st, &ctl->error, FRB_TIMEOUT, ctl->bar);
+        launch_dep(k_fr_place, dim3(152 * 4), dim3(256), 0, st, a, row_start, xyz, pulse, view_off);
+        launches = 3;   // recognition, the scan of the row counts, the placement
         cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? ET_OK : cuda_fail(e, "front-end launch");
     }
@@ -574,13 +464,10 @@ struct FramesRT {
             if (e != cudaSuccess) return cuda_fail(e, "raw frame upload");
             d_raw = (const unsigned char *)g_raw.base;
         }
-        if (want == 0) want = 65536;
-        const u64 guess = std::max<u64>(65536, (u64)nv * p.depth * p.height * p.width / 2000);
-        want = std::max(want, guess);
-        if (cap < want || view_count == nullptr || (size_t)V + 1 > last_views) {
+        want = std::max(want, std::max<u64>(65536, (u64)nv * p.depth * p.height * p.width / 2000));
+        if (cap < want || (size_t)V > last_views) {
             et_status s = reserve_out(std::max(want, cap));
             if (s != ET_OK) return s;
-            last_views = (size_t)V + 1;
         }
         et_status s = enqueue(st);
         if (s != ET_OK) return s;
