@@ -135,6 +135,17 @@ struct Out {
     int *long_tracks;    // tracks whose members are sorted on their own
 };
 
+// Page-locked host memory that the last kernel of a run writes: the control
+// block, and the results where they are small (each part 16-byte aligned).
+constexpr u32 STAGE_TRACKS = 1024, STAGE_MEMBERS = 16384, STAGE_VIEWS = 1024;
+struct Stage {
+    Ctl ctl;
+    u32 whole, pad[3];   // the results below are complete
+    alignas(16) unsigned char tracks[64 * STAGE_TRACKS];
+    alignas(16) int members[STAGE_MEMBERS];
+    alignas(16) long long view_trk[STAGE_VIEWS + 2];
+};
+
 __device__ __forceinline__ int view_of(const long long *goff, int V, long long g) {
     int lo = 0, hi = V - 1;
     while (lo < hi) {

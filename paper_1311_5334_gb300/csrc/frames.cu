@@ -72,6 +72,16 @@ struct FrArgs {
     u32 *row_head;
 };
 
+// Page-locked host memory that the last kernel of a run writes (as Stage of the
+// tracking): control block, view offsets and grains where they are few.
+constexpr u32 FSTAGE_GRAINS = 16384, FSTAGE_VIEWS = 1024;
+struct FrStage {
+    FrCtl ctl;
+    alignas(16) u32 view_off[FSTAGE_VIEWS + 4];
+    alignas(16) int xyz[3 * FSTAGE_GRAINS];
+    alignas(16) int pulse[FSTAGE_GRAINS];
+};
+
 __device__ __forceinline__ int filt(int raw, int g, int t) {
     const int v = min(255, ((255 - raw) * g + 64) >> 7);
     return max(0, v - t);
@@ -292,6 +302,21 @@ __global__ void k_fr_place(FrArgs a, const u32 *row_start, int *xyz, int *pulse,
     }
 }
 
+// Control block, view offsets and, where they are few, the grains into
+// page-locked host memory (16-byte stores in order), for a fetch without device
+// copies.
+__global__ void k_fr_publish(FrArgs a, const int *xyz, const int *pulse, const u32 *view_off, FrStage *st) {
+    griddep_launch();
+    griddep_wait();
+    const u32 tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+    if (tid == 0) st->ctl = *a.ctl;
+    for (u32 v = tid; v <= min((u32)a.V, FSTAGE_VIEWS); v += stride) st->view_off[v] = view_off[v];
+    const u64 n = min(a.ctl->n_grains, a.cap);
+    if (n > FSTAGE_GRAINS) return;
+    for (u32 i = tid; i < (3 * (u32)n + 3) / 4; i += stride) ((uint4 *)st->xyz)[i] = ((const uint4 *)xyz)[i];
+    for (u32 i = tid; i < ((u32)n + 3) / 4; i += stride) ((uint4 *)st->pulse)[i] = ((const uint4 *)pulse)[i];
+}
+
 }  // namespace
 
 // The front end of one camera (geometry and calibration) with its device buffers.
@@ -319,6 +344,7 @@ struct FramesRT {
     bool handoff_pending = false;
     bool ran = false, settled = false;
     FrCtl hctl{};
+    FrStage *stage = nullptr;   // null: results are copied by the fetch
     et_status run_status = ET_OK;
     float kernel_ms = 0.0f, run_ms = 0.0f;
 
@@ -329,6 +355,7 @@ struct FramesRT {
         for (auto &e : ev)
             if (e) cudaEventDestroy(e);
         if (handoff) cudaEventDestroy(handoff);
+        ctx->give_stage(1, stage);
         g_tab.release(ctx);
         g_raw.release(ctx);
         g_out.release(ctx);
@@ -356,6 +383,7 @@ struct FramesRT {
         cal = (unsigned short *)(cut + tb);
         if (!g_ctl.reserve(ctx, sizeof(FrCtl))) return fail(ET_ERR_OOM, "control block");
         ctl = (FrCtl *)g_ctl.base;
+        stage = (FrStage *)ctx->take_stage(1, sizeof(FrStage));
         return ET_OK;
     }
 
@@ -444,7 +472,8 @@ struct FramesRT {
         cudaEventRecord(ev[2], st);
         exclusive_scan_u32(row_count, row_start, (long long)rows(), temp, st, &ctl->error, FRB_TIMEOUT, ctl->bar);
         launch_dep(k_fr_place, dim3(152 * 4), dim3(256), 0, st, a, row_start, xyz, pulse, view_off);
-        launches = 3;   // recognition, the scan of the row counts, the placement
+        if (stage) launch_dep(k_fr_publish, dim3(16), dim3(512), 0, st, a, (const int *)xyz, (const int *)pulse, (const u32 *)view_off, stage);
+        launches = stage ? 4 : 3;   // recognition, the scan of the row counts, placement, publication
         cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? ET_OK : cuda_fail(e, "front-end launch");
     }
@@ -486,7 +515,8 @@ struct FramesRT {
         for (int attempt = 0; attempt < 4; ++attempt) {
             cudaError_t e = cudaEventSynchronize(ev[3]);
             if (e != cudaSuccess) return run_status = cuda_fail(e, "front-end run");
-            e = cudaMemcpy(&hctl, ctl, sizeof(FrCtl), cudaMemcpyDeviceToHost);
+            if (stage) hctl = stage->ctl;
+            else e = cudaMemcpy(&hctl, ctl, sizeof(FrCtl), cudaMemcpyDeviceToHost);
             if (e != cudaSuccess) return run_status = cuda_fail(e, "control block read");
             if (hctl.error & FRB_TIMEOUT) {
                 settled = true;
@@ -512,6 +542,17 @@ struct FramesRT {
     }
 
     u64 n_grains() const { return std::min(hctl.n_grains, cap); }
+
+    // View offsets of the settled run.
+    et_status offsets(std::vector<u32> &off) const {
+        off.resize((size_t)V + 1);
+        if (stage && V <= (int)FSTAGE_VIEWS) {
+            memcpy(off.data(), stage->view_off, sizeof(u32) * off.size());
+            return ET_OK;
+        }
+        const cudaError_t e = cudaMemcpy(off.data(), view_off, sizeof(u32) * off.size(), cudaMemcpyDeviceToHost);
+        return e == cudaSuccess ? ET_OK : cuda_fail(e, "view offsets");
+    }
 };
 
 }  // namespace et
@@ -598,11 +639,17 @@ et_status et_frames_fetch(et_frames *fr, int64_t *view_offsets, int32_t *xyz, in
     *n_grains = n;
     if (n > 0 && (!xyz || cap < n)) return fail(ET_ERR_CAPACITY, "need room for %lld grains", (long long)n);
     cudaError_t e = cudaSuccess;
-    if (n > 0) e = cudaMemcpy(xyz, fr->xyz, sizeof(int32_t) * 3 * (size_t)n, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess && n > 0 && pulse) e = cudaMemcpy(pulse, fr->pulse, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost);
+    if (fr->stage && n <= (int64_t)FSTAGE_GRAINS) {
+        if (n > 0) memcpy(xyz, fr->stage->xyz, sizeof(int32_t) * 3 * (size_t)n);
+        if (n > 0 && pulse) memcpy(pulse, fr->stage->pulse, sizeof(int32_t) * (size_t)n);
+    } else {
+        if (n > 0) e = cudaMemcpy(xyz, fr->xyz, sizeof(int32_t) * 3 * (size_t)n, cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess && n > 0 && pulse) e = cudaMemcpy(pulse, fr->pulse, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost);
+    }
     if (e == cudaSuccess && view_offsets) {
-        std::vector<u32> off((size_t)fr->V + 1);
-        e = cudaMemcpy(off.data(), fr->view_off, sizeof(u32) * off.size(), cudaMemcpyDeviceToHost);
+        std::vector<u32> off;
+        s = fr->offsets(off);
+        if (s != ET_OK) return s;
         for (size_t i = 0; i < off.size(); ++i) view_offsets[i] = off[i];
     }
     return e == cudaSuccess ? ET_OK : cuda_fail(e, "grain download");
@@ -616,9 +663,9 @@ et_status et_frames_to_batch(et_frames *fr, et_batch *batch, void *stream) {
     cudaSetDevice(fr->ctx->device);
     et_status s = fr->settle();
     if (s != ET_OK) return s;
-    std::vector<u32> off((size_t)fr->V + 1);
-    cudaError_t e = cudaMemcpy(off.data(), fr->view_off, sizeof(u32) * off.size(), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "view offsets");
+    std::vector<u32> off;
+    s = fr->offsets(off);
+    if (s != ET_OK) return s;
     std::vector<int64_t> off64(off.begin(), off.end());
     cudaStream_t st = stream ? (cudaStream_t)stream : fr->ctx->stream;
     if (batch->ran) cudaEventSynchronize(batch->done);

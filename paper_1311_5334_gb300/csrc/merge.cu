@@ -688,6 +688,25 @@ __global__ void __launch_bounds__(LONG_T) k_long_members(Batch b, Work w, Out o)
     }
 }
 
+// The run's control block and small results into page-locked host memory, so
+// that the caller's fetch waits once and copies on the host: a device copy
+// after the run costs about 10 us each, and a fetch took five of them.
+__global__ void k_publish(Batch b, Out o, Stage *st) {
+    griddep_launch();
+    griddep_wait();
+    const u32 t = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+    const Ctl *ctl = b.ctl;
+    for (u32 i = t; i < sizeof(Ctl) / sizeof(u32); i += nth) ((u32 *)&st->ctl)[i] = ((const u32 *)ctl)[i];
+    const bool whole = !(ctl->error & (ERRB_INPUT_MASK | ERRB_OVF_MASK | ERRB_TIMEOUT)) && ctl->n_acc <= STAGE_TRACKS &&
+                       ctl->n_out_members <= STAGE_MEMBERS && b.V <= (int)STAGE_VIEWS;
+    if (t == 0) st->whole = whole ? 1u : 0u;
+    if (!whole) return;
+    const u32 nt = (u32)ctl->n_acc, nm = (u32)ctl->n_out_members;
+    for (u32 i = t; i < nt * 4; i += nth) ((uint4 *)st->tracks)[i] = ((const uint4 *)o.tracks)[i];
+    for (u32 i = t; i < nm; i += nth) st->members[i] = o.out_members[i];
+    for (u32 i = t; i <= (u32)b.V; i += nth) st->view_trk[i] = o.view_trk[i];
+}
+
 unsigned sm_count() {
     static int sms = 0;
     if (!sms) {
@@ -724,6 +743,10 @@ cudaError_t launch_merge_coop(const Batch &b, const Work &w, int grid, cudaStrea
     Work ww = w;
     void *args[] = {&bb, &ww};
     return cudaLaunchCooperativeKernel((const void *)k_merge, dim3(grid), dim3(MT), args, 0, st);
+}
+
+void launch_publish(const Batch &b, const Out &o, Stage *st_host, cudaStream_t st) {
+    launch_dep(k_publish, dim3(8), dim3(512), 0, st, b, o, st_host);
 }
 
 const u32 *launch_cand_order(const Batch &b, const Work &w, Out &o, u64 window, void *temp, cudaStream_t st) {

@@ -14,6 +14,7 @@ namespace et {
 
 cudaError_t launch_merge_coop(const Batch &b, const Work &w, int grid, cudaStream_t st);
 void launch_output(const Batch &b, const Work &w, Out &o, long long acc_cap, void *temp, cudaStream_t st);
+void launch_publish(const Batch &b, const Out &o, Stage *st_host, cudaStream_t st);
 
 static thread_local std::string g_last_error;
 
@@ -58,6 +59,41 @@ void Ctx::dfree(void *p) {
     if (!p) return;
     if (free_fn) free_fn(p, user);
     else cudaFree(p);
+}
+
+// Page-locked memory of one kind (0: Stage, 1: the front end's), null if there is none.
+void *Ctx::take_stage(int kind, size_t bytes) {
+    {
+        std::lock_guard<std::mutex> g(stage_mu);
+        if (!stages[kind].empty()) {
+            void *p = stages[kind].back();
+            stages[kind].pop_back();
+            return p;
+        }
+    }
+    void *p = nullptr;
+    if (cudaHostAlloc(&p, bytes, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+
+void Ctx::give_stage(int kind, void *p) {
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> g(stage_mu);
+        if (stages[kind].size() < STAGE_POOL) {
+            stages[kind].push_back(p);
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
+Ctx::~Ctx() {
+    for (auto &k : stages)
+        for (void *p : k) cudaFreeHost(p);
 }
 
 // ---------------------------------------------------------------- groups
@@ -123,6 +159,7 @@ BatchRT::BatchRT(Ctx *c, const et_params &pp) : ctx(c), p(pp) {
 }
 
 BatchRT::~BatchRT() {
+    ctx->give_stage(0, stage);
     if (gexec) cudaGraphExecDestroy(gexec);
     if (done) cudaEventDestroy(done);
     for (cudaEvent_t &e : ev)
@@ -516,6 +553,7 @@ unsigned long long BatchRT::graph_signature() const {
     mix((unsigned long long)tune.wait_polls);
     mix((unsigned long long)tune.ticket_origins);
     mix((unsigned long long)tune.assoc_window);
+    mix((unsigned long long)(uintptr_t)stage);
     return h;
 }
 
@@ -551,6 +589,7 @@ et_status BatchRT::load(const int32_t *xyz, const int64_t *offsets, int nv, bool
     estimate_caps();
     et_status s = reserve();
     if (s != ET_OK) return s;
+    if (!stage) stage = (Stage *)ctx->take_stage(0, sizeof(Stage));
     cudaError_t e = cudaMemcpyAsync(goff, goff_h.data(), sizeof(long long) * (V + 1), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && N > 0)
         e = cudaMemcpyAsync(xyz_in, xyz, sizeof(int) * 3 * (size_t)N,
@@ -703,6 +742,7 @@ et_status BatchRT::enqueue(cudaStream_t st, bool record) {
     } else {
         cudaMemsetAsync(view_trk, 0, sizeof(long long) * (V + 1), st);
     }
+    if (stage) launch_publish(b, o, stage, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "kernel launch");
     return ET_OK;
@@ -751,6 +791,10 @@ et_status BatchRT::find(cudaStream_t st, bool use_graph) {
 et_status BatchRT::read_ctl(Ctl &h) {
     cudaError_t e = cudaEventSynchronize(done);
     if (e != cudaSuccess) return cuda_fail(e, "wait for the view");
+    if (stage) {
+        memcpy(&h, &stage->ctl, sizeof(Ctl));
+        return ET_OK;
+    }
     e = cudaMemcpy(&h, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "read control block");
     return ET_OK;
@@ -792,6 +836,13 @@ et_status BatchRT::fetch(int64_t *view_off, et_track *out, int64_t cap, int64_t 
     if (n_members) *n_members = nm;
     if ((nt > 0 && (!out || cap < nt)) || (nm > 0 && (!mem || mcap < nm)))
         return fail(ET_ERR_CAPACITY, "need %lld tracks / %lld members", (long long)nt, (long long)nm);
+    if (stage && stage->whole) {
+        if (nt > 0) memcpy(out, stage->tracks, sizeof(et_track) * nt);
+        if (nm > 0) memcpy(mem, stage->members, sizeof(int) * nm);
+        if (view_off)
+            for (int v = 0; v <= V; ++v) view_off[v] = stage->view_trk[v];
+        return ET_OK;
+    }
     cudaError_t e = cudaSuccess;
     if (nt > 0) e = cudaMemcpy(out, tracks, sizeof(et_track) * nt, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess && nm > 0) e = cudaMemcpy(mem, out_members, sizeof(int) * nm, cudaMemcpyDeviceToHost);

@@ -1,5 +1,6 @@
 // runtime.h -- host-side objects behind the C ABI (include/et.h).
 #pragma once
+#include <mutex>
 #include <vector>
 
 #include "common.cuh"
@@ -35,6 +36,13 @@ struct Ctx {
     et_alloc_fn alloc = nullptr;
     et_free_fn free_fn = nullptr;
     void *user = nullptr;
+    // page-locked stages given back by batches and front ends, at most STAGE_POOL
+    static constexpr size_t STAGE_POOL = 16;
+    std::mutex stage_mu;
+    std::vector<void *> stages[2];
+    void *take_stage(int kind, size_t bytes);
+    void give_stage(int kind, void *p);
+    ~Ctx();
     void *dalloc(size_t bytes);
     void dfree(void *p);
 };
@@ -103,6 +111,7 @@ struct BatchRT {
     cudaStream_t run_stream = nullptr;
     bool loaded = false, ran = false;
     Ctl hctl{};
+    Stage *stage = nullptr;   // null: results are copied by the fetch
     cudaGraphExec_t gexec = nullptr;
     unsigned long long graph_key = 0;
     // profiling
