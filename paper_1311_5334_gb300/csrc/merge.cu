@@ -55,11 +55,62 @@ constexpr unsigned long long BARRIER_SPIN_LIMIT = 1ull << 24;  // x ~128 ns slee
 
 __device__ __forceinline__ u32 ld_cg_u32(const u32 *p) { return __ldcg(p); }
 
-// Candidates per block in use: the association keeps one block per MT / 32
-// candidates (one candidate per warp, whose dependent loads are the round's
-// latency), so a short candidate list runs on few blocks whose barriers are
-// cheap, a long one on the whole grid.
+// Candidates per block in use: a short candidate list runs on few blocks, whose
+// barriers are cheap, a long one on the whole grid.
 constexpr u64 MERGE_CANDS_PER_BLOCK = MT / 32;
+
+// Up to four candidates of at most 32 grains (cnt 0: none), or one longer one.
+struct Four {
+    int c[4];
+    u32 cnt[4];
+    u64 m0[4], key[4];
+    bool lng;
+};
+
+// Calls f for the undecided candidates of this warp's share of the list (of
+// the window's candidates in order, without one).  The lanes read the states,
+// places and keys of 32 candidates at once, and candidates of at most 32 grains
+// are handed out four at a time, so that the dependent reads of one (members,
+// owners, keys; all from L2) overlap those of the others: a round over the 34k
+// candidates of a 28k-grain view took 29 us one candidate at a time.
+template <class F>
+__device__ __forceinline__ void for_candidates(const Work &w, const int *list, const u32 *corder, u64 w0, long long nl,
+                                               long long gwarp, long long nwarps, F &&f) {
+    const int lane = threadIdx.x & 31;
+    for (long long i0 = gwarp; i0 < nl; i0 += 32 * nwarps) {
+        const long long i = i0 + lane * nwarps;
+        int c = 0;
+        u32 cnt = 0;
+        u64 m0 = 0, key = 0;
+        bool open = false;
+        if (i < nl) {
+            // lists and states are rewritten by other SMs between rounds: read through L2
+            c = list ? __ldcg(&list[i]) : (int)(corder ? (long long)corder[w0 + i] : i);
+            cnt = w.c_cnt[c];
+            m0 = w.c_moff[c];
+            key = w.c_key[c];
+            open = __ldcg(&w.c_state[c]) == CS_UNDECIDED;
+        }
+        const unsigned longs = __ballot_sync(0xffffffffu, open && cnt > 32);
+        unsigned todo = __ballot_sync(0xffffffffu, open);
+        while (todo) {
+            Four q;
+            q.lng = (longs >> (__ffs(todo) - 1)) & 1u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int src = todo ? __ffs(todo) - 1 : 0;
+                const bool take = todo && (k == 0 || (!q.lng && !((longs >> src) & 1u)));
+                q.c[k] = __shfl_sync(0xffffffffu, c, src);
+                const u32 n = __shfl_sync(0xffffffffu, cnt, src);
+                q.m0[k] = __shfl_sync(0xffffffffu, m0, src);
+                q.key[k] = __shfl_sync(0xffffffffu, key, src);
+                q.cnt[k] = take ? n : 0u;
+                if (take) todo &= todo - 1;
+            }
+            f(q);
+        }
+    }
+}
 
 // Angle cut (ET_FLAG_ANGLE_CUT): keep a track iff
 //     nhits >= cut_base + cut_slope * min(tan theta, cut_tmax),
@@ -85,7 +136,7 @@ __device__ __forceinline__ void take_track(const Batch &b, const Work &w, long l
     w.acc[atomicAdd(&b.ctl->n_acc, 1ull)] = (int)c;
 }
 
-__global__ void __launch_bounds__(MT, 4) k_merge(Batch b, Work w) {
+__global__ void __launch_bounds__(MT, 3) k_merge(Batch b, Work w) {
     griddep_launch();
     griddep_wait();
     Ctl *ctl = b.ctl;
@@ -118,49 +169,52 @@ __global__ void __launch_bounds__(MT, 4) k_merge(Batch b, Work w) {
         if (blockIdx.x == 0 && threadIdx.x == 0) ctl->ncl[(round + 1) & 1] = 0;
         // ---- phase 1: reject hopeless candidates, post keys on unused grains
         u32 my_active = 0;
-        for (long long i = gwarp; i < nl; i += nwarps) {
-            // lists and states are rewritten by other SMs between rounds: read through L2
-            const long long c = list ? __ldcg(&list[i]) : (corder ? (long long)corder[w0 + i] : i);
-            if (__ldcg(&w.c_state[c]) != CS_UNDECIDED) continue;
-            const u64 m0 = w.c_moff[c], m1 = m0 + w.c_cnt[c];
-            if (m1 - m0 <= 32) {   // one chunk: member and its state stay in registers
-                const u64 m = m0 + lane;
-                const bool in = m < m1;
-                const int g = in ? w.members[m] : 0;
-                if (in && !first) Bp[g] = ~0ull;
-                const bool fr = in && __ldcg(&w.owner[g]) < 0;
-                const u32 nfree = __popc(__ballot_sync(0xffffffffu, fr));
+        for_candidates(w, list, corder, w0, nl, gwarp, nwarps, [&](const Four &f) {
+            if (f.lng) {   // one candidate of more than 32 grains
+                const u64 m0 = f.m0[0], m1 = m0 + f.cnt[0];
+                u32 nfree = 0;
+                for (u64 base = m0; base < m1; base += 32) {
+                    const u64 m = base + lane;
+                    const bool in = m < m1;
+                    const int g = in ? w.members[m] : 0;
+                    if (in && !first) Bp[g] = ~0ull;   // entries this candidate posted last round
+                    const bool fr = in && __ldcg(&w.owner[g]) < 0;
+                    nfree += __popc(__ballot_sync(0xffffffffu, fr));
+                }
                 if (nfree < H) {
-                    if (lane == 0) w.c_state[c] = CS_REJECTED;
-                    continue;
+                    if (lane == 0) w.c_state[f.c[0]] = CS_REJECTED;
+                    return;
                 }
-                if (fr) atomicMin(&B[g], w.c_key[c]);
+                for (u64 base = m0; base < m1; base += 32) {
+                    const u64 m = base + lane;
+                    if (m < m1) {
+                        const int g = w.members[m];
+                        if (__ldcg(&w.owner[g]) < 0) atomicMin(&B[g], f.key[0]);
+                    }
+                }
                 ++my_active;
-                continue;
+                return;
             }
-            u32 nfree = 0;
-            for (u64 base = m0; base < m1; base += 32) {
-                const u64 m = base + lane;
-                const bool in = m < m1;
-                const int g = in ? w.members[m] : 0;
-                if (in && !first) Bp[g] = ~0ull;   // entries this candidate posted last round
-                const bool fr = in && __ldcg(&w.owner[g]) < 0;
-                nfree += __popc(__ballot_sync(0xffffffffu, fr));
+            int g[4];
+            bool fr[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) g[k] = lane < (int)f.cnt[k] ? w.members[f.m0[k] + lane] : -1;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (g[k] >= 0 && !first) Bp[g[k]] = ~0ull;
+                fr[k] = g[k] >= 0 && __ldcg(&w.owner[g[k]]) < 0;
             }
-            if (nfree < H) {
-                if (lane == 0) w.c_state[c] = CS_REJECTED;
-                continue;
-            }
-            const u64 key = w.c_key[c];
-            for (u64 base = m0; base < m1; base += 32) {
-                const u64 m = base + lane;
-                if (m < m1) {
-                    const int g = w.members[m];
-                    if (__ldcg(&w.owner[g]) < 0) atomicMin(&B[g], key);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (f.cnt[k] == 0) continue;   // fewer than four
+                if (__popc(__ballot_sync(0xffffffffu, fr[k])) < H) {
+                    if (lane == 0) w.c_state[f.c[k]] = CS_REJECTED;
+                } else {
+                    if (fr[k]) atomicMin(&B[g[k]], f.key[k]);
+                    ++my_active;
                 }
             }
-            ++my_active;
-        }
+        });
         if (lane == 0 && my_active) atomicAdd(&ctl->active[round & 1], my_active);
         if (!coop_barrier(ctl->bar, nb, &ctl->error, ERRB_TIMEOUT, lim)) return;
         const u32 active = ld_cg_u32(&ctl->active[round & 1]);
@@ -176,91 +230,84 @@ __global__ void __launch_bounds__(MT, 4) k_merge(Batch b, Work w) {
         int *next = w.clist[(round + 1) & 1];
         u64 *next_n = &ctl->ncl[(round + 1) & 1];
         int nkeep = 0;   // warp-uniform
-        for (long long i = gwarp; i < nl; i += nwarps) {
-            const long long c = list ? __ldcg(&list[i]) : (corder ? (long long)corder[w0 + i] : i);
-            if (__ldcg(&w.c_state[c]) != CS_UNDECIDED) continue;
-            const u64 m0 = w.c_moff[c], m1 = m0 + w.c_cnt[c];
-            const u64 key = w.c_key[c];
-            if (m1 - m0 <= 32) {   // one chunk: member and its state stay in registers
-                const u64 m = m0 + lane;
-                const bool in = m < m1;
-                const int g = in ? w.members[m] : 0;
-                const bool fr = in && __ldcg(&w.owner[g]) < 0;
-                const bool bad = fr && __ldcg(&B[g]) != key;
-                if (__any_sync(0xffffffffu, bad)) {
-                    if (lane == 0) keep[wib][nkeep] = (int)c;
-                    if (++nkeep == 32) {
-                        __syncwarp();
-                        u64 pos = 0;
-                        if (lane == 0) pos = atomicAdd(next_n, 32ull);
-                        pos = __shfl_sync(0xffffffffu, pos, 0);
-                        next[pos + lane] = keep[wib][lane];
-                        nkeep = 0;
-                        __syncwarp();
+        auto carry = [&](int c) {
+            if (lane == 0) keep[wib][nkeep] = c;
+            if (++nkeep == 32) {
+                __syncwarp();
+                u64 pos = 0;
+                if (lane == 0) pos = atomicAdd(next_n, 32ull);
+                pos = __shfl_sync(0xffffffffu, pos, 0);
+                next[pos + lane] = keep[wib][lane];
+                nkeep = 0;
+                __syncwarp();
+            }
+        };
+        auto decide = [&](int c, u32 nfree, bool accept) {   // lane 0
+            w.c_nfree[c] = nfree;
+            w.c_state[c] = accept ? CS_ACCEPTED : CS_REJECTED;
+            if (accept) take_track(b, w, c, nfree);
+        };
+        for_candidates(w, list, corder, w0, nl, gwarp, nwarps, [&](const Four &f) {
+            if (f.lng) {
+                const u64 m0 = f.m0[0], m1 = m0 + f.cnt[0], key = f.key[0];
+                u32 nfree = 0;
+                for (u64 base = m0; base < m1; base += 32) {
+                    const u64 m = base + lane;
+                    bool fr = false, bad = false;
+                    if (m < m1) {
+                        const int g = w.members[m];
+                        fr = __ldcg(&w.owner[g]) < 0;
+                        bad = fr && __ldcg(&B[g]) != key;
                     }
+                    if (__any_sync(0xffffffffu, bad)) {
+                        carry(f.c[0]);
+                        return;
+                    }
+                    nfree += __popc(__ballot_sync(0xffffffffu, fr));
+                }
+                // ready: the unused grains are exactly those where this key is the
+                // minimum; nobody else can take them any more
+                const bool accept = nfree >= H;
+                for (u64 base = m0; base < m1; base += 32) {
+                    const u64 m = base + lane;
+                    if (m < m1) {
+                        const int g = w.members[m];
+                        if (__ldcg(&w.owner[g]) < 0) {
+                            if (accept) w.owner[g] = f.c[0];
+                            B[g] = ~0ull;
+                        }
+                    }
+                }
+                if (lane == 0) decide(f.c[0], nfree, accept);
+                return;
+            }
+            // four candidates' members, owners and keys are read before any of
+            // them is decided: one that loses a grain to another of the four still
+            // sees that grain's smaller key (or the reset slot) and waits a round
+            int g[4];
+            bool fr[4], bad[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) g[k] = lane < (int)f.cnt[k] ? w.members[f.m0[k] + lane] : -1;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) fr[k] = g[k] >= 0 && __ldcg(&w.owner[g[k]]) < 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) bad[k] = fr[k] && __ldcg(&B[g[k]]) != f.key[k];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (f.cnt[k] == 0) continue;
+                if (__any_sync(0xffffffffu, bad[k])) {
+                    carry(f.c[k]);
                     continue;
                 }
-                const u32 nfree = __popc(__ballot_sync(0xffffffffu, fr));
+                const u32 nfree = __popc(__ballot_sync(0xffffffffu, fr[k]));
                 const bool accept = nfree >= H;
-                if (fr) {
-                    if (accept) w.owner[g] = (int)c;
-                    B[g] = ~0ull;
+                if (fr[k]) {
+                    if (accept) w.owner[g[k]] = f.c[k];
+                    B[g[k]] = ~0ull;
                 }
-                if (lane == 0) {
-                    w.c_nfree[c] = nfree;
-                    w.c_state[c] = accept ? CS_ACCEPTED : CS_REJECTED;
-                    if (accept) take_track(b, w, c, nfree);
-                }
-                continue;
+                if (lane == 0) decide(f.c[k], nfree, accept);
             }
-            bool ready = true;
-            u32 nfree = 0;
-            for (u64 base = m0; base < m1; base += 32) {
-                const u64 m = base + lane;
-                bool fr = false, bad = false;
-                if (m < m1) {
-                    const int g = w.members[m];
-                    fr = __ldcg(&w.owner[g]) < 0;
-                    bad = fr && __ldcg(&B[g]) != key;
-                }
-                if (__any_sync(0xffffffffu, bad)) {
-                    ready = false;
-                    break;
-                }
-                nfree += __popc(__ballot_sync(0xffffffffu, fr));
-            }
-            if (!ready) {
-                if (lane == 0) keep[wib][nkeep] = (int)c;
-                if (++nkeep == 32) {
-                    __syncwarp();
-                    u64 pos = 0;
-                    if (lane == 0) pos = atomicAdd(next_n, 32ull);
-                    pos = __shfl_sync(0xffffffffu, pos, 0);
-                    next[pos + lane] = keep[wib][lane];
-                    nkeep = 0;
-                    __syncwarp();
-                }
-                continue;
-            }
-            // ready: the unused grains are exactly those where this key is the
-            // minimum; nobody else can take them any more
-            const bool accept = nfree >= H;
-            for (u64 base = m0; base < m1; base += 32) {
-                const u64 m = base + lane;
-                if (m < m1) {
-                    const int g = w.members[m];
-                    if (__ldcg(&w.owner[g]) < 0) {
-                        if (accept) w.owner[g] = (int)c;
-                        B[g] = ~0ull;
-                    }
-                }
-            }
-            if (lane == 0) {
-                w.c_nfree[c] = nfree;
-                w.c_state[c] = accept ? CS_ACCEPTED : CS_REJECTED;
-                if (accept) take_track(b, w, c, nfree);
-            }
-        }
+        });
         if (nkeep > 0) {
             __syncwarp();
             u64 pos = 0;
