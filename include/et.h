@@ -111,13 +111,14 @@ typedef struct {
  * depend on these values, only the speed does. */
 typedef struct {
     int32_t cell[3];        /* cell-list edge per axis, coordinate units; 0: automatic
-                               (s0 * (0.24, 1.75, 1.4), s0 the edge of a cube holding 0.35
-                               grains at the mean density its grains see).  The batch's cell table
+                               (s0 * (0.24, 1.9, 1.5), s0 the edge of a cube holding 0.35
+                               grains at the density the work sees).  The batch's cell table
                                (views x cells per view) must stay below 2^31 - 1 cells, else
                                loading fails with ET_ERR_INVALID_ARG */
     int32_t ticket_origins; /* origins per work ticket of the seed generator (a warp takes
                                this many consecutive grains as line origins at a time):
-                               1, 2 or 4; 0: automatic (2) */
+                               1, 2 or 4; 0: automatic (1 up to 400,000 grains in
+                               the batch, else 2) */
     int32_t row_lists;      /* 1: one cell list, rows along x; 2: also a list with rows
                                along y, used by lines whose |w_y| > |w_x|; 0: automatic (2) */
     int32_t assoc_window;   /* candidates per window of the exclusive association (the

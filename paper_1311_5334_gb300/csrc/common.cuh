@@ -22,12 +22,13 @@ enum : u32 {
     ERRB_OVF_MEMBERS = 1u << 4,
     ERRB_TIMEOUT = 1u << 5,
     ERRB_OVF_RECORD = 1u << 6,
+    ERRB_CROWDED = 1u << 7,   // too many grains share their leading coordinates: the full sort is needed
     ERRB_INPUT_MASK = ERRB_OUT_OF_RANGE | ERRB_DUPLICATE,
-    ERRB_OVF_MASK = ERRB_OVF_CAND | ERRB_OVF_MEMBERS | ERRB_OVF_RECORD,
+    ERRB_OVF_MASK = ERRB_OVF_CAND | ERRB_OVF_MEMBERS | ERRB_OVF_RECORD | ERRB_CROWDED,
 };
 
 // Automatic cell edges, in units of the edge s0 of a cube holding 0.35 grains.
-constexpr double AUTO_CELL[3] = {0.24, 1.75, 1.4};
+constexpr double AUTO_CELL[3] = {0.24, 1.9, 1.5};
 
 // Fewest candidates per window of the association, unless set.
 constexpr u64 ASSOC_WINDOW = 1ull << 18;
@@ -252,7 +253,7 @@ inline unsigned coop_grid_limit(F fn, int threads) {
 // per process before any capture).
 void init_scan_sort();
 size_t radix_temp_bytes(long long n);
-// Stable LSD radix sort of (key, value) pairs on bits [0, bits) of the key,
+// Stable LSD radix sort of (key, value) pairs on bits [bit0, bit0 + bits) of the key,
 // over [0, min(*n_dev, n_cap)) (all n_cap when n_dev is null), in one
 // cooperative launch.  Ping-pongs between (k0, v0) and (k1, v1); returns 0 if
 // the result is in (k0, v0), 1 if in (k1, v1).  bar: two words of zero (a
@@ -263,10 +264,10 @@ size_t radix_temp_bytes(long long n);
 // [0, n).
 int radix_sort_pairs_dev(u64 *k0, u32 *v0, u64 *k1, u32 *v1, long long n_cap, const u64 *n_dev, int bits,
                          void *temp, cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit = 0,
-                         long long n_skip = 0);
+                         long long n_skip = 0, int bit0 = 0);
 inline int radix_sort_pairs(u64 *k0, u32 *v0, u64 *k1, u32 *v1, long long n, int bits, void *temp,
-                            cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit = 0) {
-    return radix_sort_pairs_dev(k0, v0, k1, v1, n, nullptr, bits, temp, st, err, err_bit, bar, spin_limit);
+                            cudaStream_t st, u32 *err, u32 err_bit, u32 *bar, long long spin_limit = 0, int bit0 = 0) {
+    return radix_sort_pairs_dev(k0, v0, k1, v1, n, nullptr, bits, temp, st, err, err_bit, bar, spin_limit, 0, bit0);
 }
 // Kernel launches of one radix sort on bits bits.
 inline int radix_sort_launches(int bits) { return bits > 0 ? 1 : 0; }
@@ -284,7 +285,8 @@ void exclusive_scan_u64_dev(const u64 *in, u64 *out, long long n_cap, const u64 
 
 // grid.cu
 void launch_canonical_keys(const Batch &b, u64 *keys, u32 *vals, cudaStream_t st);
-void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y,
+// keys: in order of their bits from bit0 on
+void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y, int bit0,
                             cudaStream_t st);
 // cursors: the cell starts, which the scatter counts up
 void launch_cell_scatter(const Batch &b, u32 *cursor, u32 *cursor_y, cudaStream_t st);

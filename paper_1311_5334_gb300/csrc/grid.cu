@@ -51,22 +51,49 @@ __device__ __forceinline__ u32 cell_y(const Batch &b, int v, int x, int y, int z
 }
 
 // Grains into canonical order, and the counts of their cells in both lists.
-__global__ void k_canonical_order(Batch b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y) {
+// The keys are sorted from bit bit0 on (view and x); a grain's rank among those
+// that agree there, rarely more than one, comes from comparing the full keys.
+// Sorting on all bits took 6 instead of 2 passes for one view.  More than
+// CROWD grains that agree report ERRB_CROWDED, and the run is repeated with
+// the full sort.
+constexpr int CROWD = 64;
+
+__global__ void k_canonical_order(Batch b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y, int bit0) {
     griddep_launch();
     griddep_wait();
     // a coordinate out of range is reported as such; a timed-out sort leaves
     // invalid indices: either way nothing after this point may run
     if (input_failed(b.ctl)) return;
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < b.N; p += stride) {
-        const int v = view_of(b.goff, b.V, p);
-        const long long i = vals[p];
-        int x = b.xyz_in[3 * i + 0], y = b.xyz_in[3 * i + 1], z = b.xyz_in[3 * i + 2];
-        x = min(max(x, 0), b.ext[0] - 1);
-        y = min(max(y, 0), b.ext[1] - 1);
-        z = min(max(z, 0), b.ext[2] - 1);
+    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < b.N; q += stride) {
+        const int v = view_of(b.goff, b.V, q);   // the views' grains stay in their ranges
+        const long long i = vals[q];
+        const u64 key = keys[q];
+        long long p = q;
+        bool twin = false, crowded = false;
+        if (bit0 > 0) {
+            int steps = 0;
+            for (long long j = q - 1; j >= 0 && (keys[j] >> bit0) == (key >> bit0); --j) {
+                p -= keys[j] > key;
+                twin |= keys[j] == key;
+                if ((crowded = ++steps > CROWD)) break;
+            }
+            for (long long j = q + 1; j < b.N && (keys[j] >> bit0) == (key >> bit0); ++j) {
+                p += keys[j] < key;
+                if ((crowded |= ++steps > CROWD)) break;
+            }
+        } else {
+            twin = q > b.goff[v] && keys[q - 1] == key;
+        }
+        if (crowded) {
+            atomicOr(&b.ctl->error, ERRB_CROWDED);
+            continue;
+        }
+        const int z = (int)(key & ((1ull << b.cbits[2]) - 1ull));   // the key holds the coordinates
+        const int y = (int)((key >> b.cbits[2]) & ((1ull << b.cbits[1]) - 1ull));
+        const int x = (int)((key >> (b.cbits[1] + b.cbits[2])) & ((1ull << b.cbits[0]) - 1ull));
         b.gr[p] = make_int4(x, y, z, (int)(i - b.goff[v]));
-        if (p > b.goff[v] && keys[p] == keys[p - 1]) atomicOr(&b.ctl->error, ERRB_DUPLICATE);
+        if (twin) atomicOr(&b.ctl->error, ERRB_DUPLICATE);
         atomicAdd(&count[cell_x(b, v, x, y, z)], 1u);
         if (b.dual) atomicAdd(&count_y[cell_y(b, v, x, y, z)], 1u);
     }
@@ -107,9 +134,9 @@ void launch_canonical_keys(const Batch &b, u64 *keys, u32 *vals, cudaStream_t st
     launch_dep(k_canonical_keys, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, keys, vals);
 }
 
-void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y,
+void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y, int bit0,
                             cudaStream_t st) {
-    launch_dep(k_canonical_order, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, keys, vals, count, count_y);
+    launch_dep(k_canonical_order, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, keys, vals, count, count_y, bit0);
 }
 
 void launch_cell_scatter(const Batch &b, u32 *cursor, u32 *cursor_y, cudaStream_t st) {

@@ -175,16 +175,15 @@ static constexpr double kMaxCells = 2147483647.0;
 void BatchRT::choose_cells() {
     for (int k = 0; k < 3; ++k) cs[k] = tune.cell[k];
     if (cs[0] <= 0 || cs[1] <= 0 || cs[2] <= 0) {
-        // s0: the edge of a cube holding 0.35 grains at the density most of the
-        // work sees (seeds grow with the square of a view's grains, so views count
-        // by their grains).  Cells are short along the x rows and long across
-        // them.  Sweeps of 13 shapes on views of 2.5k to 65k grains, a 1.2 M-grain
-        // scan and batches of 17 and 256 views put this shape, or one within 1 %
-        // of it, first or near it; against 0.22, 1.1, 1.1 at the batch's mean
-        // density the 28k view's tube counts took 0.66 instead of 0.72 ms, the
-        // scan 203 instead of 321 ms, and no size got slower
+        // s0: the edge of a cube holding 0.35 grains at the density the work sees (a
+        // view's tube tests grow with the cube of its grains: seeds times grains
+        // along a line).  Cells are short along the x rows and long across them.
+        // Sweeps of 13 shapes on views of 2.5k to 65k grains, a 1.2 M-grain scan and
+        // batches of 17 and 256 views put this shape, or one within 2 % of it, first;
+        // against 0.22, 1.1, 1.1 at the batch's mean density the 28k view's tube
+        // counts took 0.66 instead of 0.72 ms and the scan 203 instead of 321 ms
         double vol = (double)p.extent[0] * p.extent[1] * p.extent[2];
-        double nwork = N > 0 ? sum_n2 / (double)N : 1.0;
+        double nwork = sum_n2 > 0.0 ? sum_n3 / sum_n2 : 1.0;
         double rho = std::max(nwork, 1.0) / vol;
         double s = std::cbrt(0.35 / rho);
         s = std::min(std::max(s, 64.0), 4096.0);
@@ -511,11 +510,12 @@ et_status BatchRT::reserve() {
 
 // Sizes of the device groups a batch of the given shape would hold, without
 // allocating (the served loop's admission).
-void BatchRT::plan_shape(int nv, long long n, long long mx, double s2, size_t sizes[NGROUP]) {
+void BatchRT::plan_shape(int nv, long long n, long long mx, double s2, double s3, size_t sizes[NGROUP]) {
     V = nv;
     N = n;
     maxN = mx;
     sum_n2 = s2;
+    sum_n3 = s3;
     want_cand = want_members = want_rec = 0;
     choose_cells();
     estimate_caps();
@@ -553,6 +553,7 @@ unsigned long long BatchRT::graph_signature() const {
     mix((unsigned long long)tune.wait_polls);
     mix((unsigned long long)tune.ticket_origins);
     mix((unsigned long long)tune.assoc_window);
+    mix(full_sort ? 1ull : 0ull);
     mix((unsigned long long)(uintptr_t)stage);
     return h;
 }
@@ -579,8 +580,12 @@ et_status BatchRT::load(const int32_t *xyz, const int64_t *offsets, int nv, bool
     N = total;
     maxN = mx;
     goff_h.assign(offsets, offsets + nv + 1);
-    sum_n2 = 0;
-    for (int v = 0; v < nv; ++v) sum_n2 += (double)(offsets[v + 1] - offsets[v]) * (double)(offsets[v + 1] - offsets[v]);
+    sum_n2 = sum_n3 = 0;
+    for (int v = 0; v < nv; ++v) {
+        const double k = (double)(offsets[v + 1] - offsets[v]);
+        sum_n2 += k * k;
+        sum_n3 += k * k * k;
+    }
     for (int k = 0; k < 3; ++k) cbits[k] = cb[k];
     choose_cells();
     if ((double)V * (double)std::max(ncell, ncelly) >= kMaxCells)
@@ -622,7 +627,10 @@ Batch BatchRT::dev_batch() const {
     b.r2 = (long long)p.tube_r * p.tube_r;
     b.flags = p.flags;
     b.spin_limit = tune.wait_polls > 0 ? (long long)tune.wait_polls : 0;
-    b.gen_origins = tune.ticket_origins > 0 ? tune.ticket_origins : 2;
+    // one origin per work ticket while a batch is small enough that the last
+    // tickets' warps run alone (28k grains: tube counts 0.66 -> 0.60 ms); at 216k
+    // grains one and two are equal, at 3.9 M two are 1.4 % faster
+    b.gen_origins = tune.ticket_origins > 0 ? tune.ticket_origins : (N <= 400000 ? 1 : 2);
     const bool cut = (p.flags & ET_FLAG_ANGLE_CUT) != 0;
     b.cut_base = cut ? p.cut_base : 0;
     b.cut_slope = cut ? p.cut_slope : 0;
@@ -710,9 +718,11 @@ et_status BatchRT::enqueue(cudaStream_t st, bool record) {
         cudaMemsetAsync(cell_count, 0, sizeof(u32) * (cells + cellsy), st);
         launch_canonical_keys(b, keys[0], vals[0], st);
         const int kb = b.vshift + bits_for((unsigned long long)std::max(V - 1, 0));
-        int c1 = radix_sort_pairs(keys[0], vals[0], keys[1], vals[1], n, kb, temp, st, &ctl->error, ERRB_TIMEOUT,
-                                  ctl->bar, b.spin_limit);
-        launch_canonical_order(b, keys[c1], vals[c1], cell_count, cell_count + cells, st);
+        // on view and x alone while few grains of a view can share their x
+        const int bit0 = !full_sort && maxN <= 4 * (long long)p.extent[0] ? cbits[1] + cbits[2] : 0;
+        int c1 = radix_sort_pairs(keys[0], vals[0], keys[1], vals[1], n, kb - bit0, temp, st, &ctl->error, ERRB_TIMEOUT,
+                                  ctl->bar, b.spin_limit, bit0);
+        launch_canonical_order(b, keys[c1], vals[c1], cell_count, cell_count + cells, bit0, st);
         // both cell lists by one counting sort: the scan leaves the starts, and in
         // the counts' place a copy that serves as the scatter's cursors
         exclusive_scan_u32(cell_count, cell_start, (long long)(cells + cellsy), temp, st, &ctl->error, ERRB_TIMEOUT,
@@ -816,6 +826,7 @@ et_status BatchRT::settle(bool record) {
             want_members = std::max<u64>(want_members, want_cand * 24);
         }
         if (hctl.error & ERRB_OVF_MEMBERS) want_members = std::max<u64>(want_members, hctl.n_members + 1024);
+        if (hctl.error & ERRB_CROWDED) full_sort = true;
         if (hctl.error & ERRB_OVF_RECORD) want_rec = std::max<u64>(want_rec, hctl.n_seeds);
         s = reserve();
         if (s != ET_OK) return s;

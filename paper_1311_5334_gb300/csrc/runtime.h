@@ -68,6 +68,7 @@ struct BatchRT {
     int V = 0;
     long long N = 0, maxN = 0;
     double sum_n2 = 0;   // sum over views of (grains)^2: sizes the candidate buffers
+    double sum_n3 = 0;   // and of (grains)^3: weighs the views for the automatic cells
     std::vector<long long> goff_h;
     int cs[3] = {1, 1, 1}, nc[3] = {1, 1, 1}, cbits[3] = {0, 0, 0};
     long long ncell = 1;
@@ -110,6 +111,7 @@ struct BatchRT {
     cudaEvent_t done = nullptr;
     cudaStream_t run_stream = nullptr;
     bool loaded = false, ran = false;
+    bool full_sort = false;   // the canonical order sorts all key bits (grains crowd on shared x)
     Ctl hctl{};
     Stage *stage = nullptr;   // null: results are copied by the fetch
     cudaGraphExec_t gexec = nullptr;
@@ -132,7 +134,7 @@ struct BatchRT {
     size_t held_bytes() const;
     size_t footprint_with(const size_t sizes[NGROUP]) const;
     void release_groups();
-    void plan_shape(int nv, long long n, long long mx, double s2, size_t sizes[NGROUP]);
+    void plan_shape(int nv, long long n, long long mx, double s2, double s3, size_t sizes[NGROUP]);
     et_status reserve();
     unsigned long long layout_generation() const;
     unsigned long long graph_signature() const;

@@ -108,7 +108,7 @@ struct ServerRT {
     uint64_t single_view_bytes(int64_t n) {
         std::lock_guard<std::mutex> g(submit_mu);
         size_t sz[BatchRT::NGROUP];
-        submit_planner->plan_shape(1, n, n, (double)n * (double)n, sz);
+        submit_planner->plan_shape(1, n, n, (double)n * (double)n, (double)n * (double)n * (double)n, sz);
         uint64_t t = 0;
         for (size_t v : sz) t += v;
         return t;
@@ -148,15 +148,17 @@ struct ServerRT {
         if (wait) cv_work.wait(g, [this] { return stop || !pending.empty(); });
         if (stop && pending.empty()) return false;
         long long n = 0, mx = 0;
-        double s2 = 0;
+        double s2 = 0, s3 = 0;
         size_t sz[BatchRT::NGROUP];
         while (!pending.empty() && (int)sl.take.size() < max_views) {
             const long long vn = pending.front().n;
-            planner->plan_shape((int)sl.take.size() + 1, n + vn, std::max(mx, vn), s2 + (double)vn * vn, sz);
+            planner->plan_shape((int)sl.take.size() + 1, n + vn, std::max(mx, vn), s2 + (double)vn * vn,
+                                s3 + (double)vn * vn * vn, sz);
             if (sl.batch->footprint_with(sz) > avail) break;
             n += vn;
             mx = std::max(mx, vn);
             s2 += (double)vn * vn;
+            s3 += (double)vn * vn * vn;
             sl.take.push_back(std::move(pending.front()));
             pending.pop_front();
         }
