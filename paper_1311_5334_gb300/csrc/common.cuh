@@ -92,7 +92,6 @@ struct Batch {
     int csy[3], ncy[3];
     float icsy[3];
     int ncelly;
-    u32 *cell_start_y;   // V * ncelly + 1
     Ctl *ctl;
 };
 

@@ -42,9 +42,8 @@ constexpr long long NA_LIST_CELLS = NA_MAX_CELLS / 2;
 constexpr size_t NA_ALIGN = 256;
 constexpr size_t na_up(size_t v) { return (v + NA_ALIGN - 1) / NA_ALIGN * NA_ALIGN; }
 constexpr size_t NA_OFF_GRAINS = 0;                                                       // u64[2 MAX_GRAINS]
-constexpr size_t NA_OFF_START = NA_OFF_GRAINS + sizeof(u64) * 2 * NA_MAX_GRAINS;          // u32[2][LIST_CELLS + 1]
-constexpr size_t NA_START_BYTES = na_up(sizeof(u32) * (NA_LIST_CELLS + 1));
-constexpr size_t NA_OFF_CURSOR = NA_OFF_START + 2 * NA_START_BYTES;                       // u32[2][LIST_CELLS]
+constexpr size_t NA_OFF_START = NA_OFF_GRAINS + sizeof(u64) * 2 * NA_MAX_GRAINS;          // u32[2 LIST_CELLS + 1]
+constexpr size_t NA_OFF_CURSOR = NA_OFF_START + na_up(sizeof(u32) * (2 * NA_LIST_CELLS + 1));   // u32[2][LIST_CELLS]
 constexpr size_t NA_OFF_CTL = NA_OFF_CURSOR + sizeof(u32) * NA_MAX_CELLS;                 // NaCtl
 constexpr size_t NA_BYTES = NA_OFF_CTL + NA_ALIGN;
 
@@ -61,13 +60,15 @@ struct NaScratch {
     NaCtl *ctl;
 };
 
-NaScratch carve(unsigned char *base) {
+// n0: cells of the first list (the second list's starts follow them)
+NaScratch carve(unsigned char *base, long long n0) {
     NaScratch s;
     s.grains = (u64 *)(base + NA_OFF_GRAINS);
     for (int l = 0; l < 2; ++l) {
-        s.start[l] = (u32 *)(base + NA_OFF_START + l * NA_START_BYTES);
         s.cursor[l] = (u32 *)(base + NA_OFF_CURSOR) + l * NA_LIST_CELLS;
     }
+    s.start[0] = (u32 *)(base + NA_OFF_START);
+    s.start[1] = s.start[0] + n0;
     s.ctl = (NaCtl *)(base + NA_OFF_CTL);
     return s;
 }
@@ -164,7 +165,8 @@ __global__ void __launch_bounds__(1024) k_na_scan(NaScratch s, int n0, int n1, u
         }
         __syncthreads();   // part is written again
     }
-    if (threadIdx.x == 0) start[n] = carry;
+    // the first list's end is the second one's first start, written by its block
+    if (threadIdx.x == 0 && list) start[n] = carry;
 }
 
 __global__ void k_na_scatter(Batch b, const int *xyz, NaScratch s) {
@@ -339,9 +341,8 @@ extern "C" et_status et_tube_count_noalloc(const int32_t *d_xyz, int64_t n, cons
     b.ncell = (int)nx;
     b.ncelly = (int)ny;
     b.dual = 1;
-    const NaScratch s = carve(base);
+    const NaScratch s = carve(base, nx);
     b.cell_start = s.start[0];
-    b.cell_start_y = s.start[1];
     b.gp = s.grains;
     cudaStream_t cst = (cudaStream_t)stream;
     const unsigned gc = (unsigned)std::min<long long>((std::max(nx, ny) + 255) / 256, 608);

@@ -643,7 +643,6 @@ Batch BatchRT::dev_batch() const {
     }
     b.ncelly = (int)ncelly;
     b.dual = dual ? 1 : 0;
-    b.cell_start_y = cell_start + (size_t)V * (size_t)ncell;
     b.vshift = cbits[0] + cbits[1] + cbits[2];
     b.rbits = std::max(1, bits_for((unsigned long long)maxN));
     b.xyz_in = xyz_in;

@@ -18,18 +18,18 @@ namespace et {
 // the round (an OR-reduction of one-hot masks and a popcount).  Line geometry
 // is resolved once into shared memory; per-line results are merged with
 // shared-memory atomics.  The geometry is the conservative cover of
-// tube_cover() (tube.cuh), with the per-slab terms hoisted.
+// tube.cuh, with the per-slab terms hoisted.
 // Cover geometry of one line, resolved once per line into eight 16-byte
 // vectors (an item loads the six it needs, a grain test the first two).  Slab t-intervals
 // are kept as (lower end at cell 0, step per cell, width) with the direction's
 // sign already folded in, so the walk needs no min/max to order their ends.
 struct __align__(16) SeedSm {
-    int4 e0;      // ax, ay, az, wx
+    int4 e0;      // a x w (three components), wx
     int4 e1;      // wy, wz, R low, R high           (R = r^2 |w|^2)
     float4 e2;    // t0, t1 (span of the line near the view), o0, excl (int bits)
     float4 e3;    // outer slab: lower base, step, width; inner cell count (int bits)
     float4 e4;    // inner slab: lower base, step, width, 1 / inner cell edge
-    float4 e5;    // inner axis: a - pad, a + pad, w, flags (int bits: 1 second list, 2 w_inner < 0, 4 w_run < 0)
+    float4 e5;    // inner axis: a - pad, a + pad, w, flags (int bits: 2 w_inner < 0, 4 w_run < 0)
     float4 e6;    // run axis: a - pad, a + pad, w, 1 / run cell edge
     int4 e7;      // run cell count, row stride of outer cell, of inner cell, view offset in the start table
 };
@@ -78,7 +78,7 @@ __device__ __forceinline__ int seed_setup(const Batch &b, int4 ga, int4 gb, int 
     const float pad = (float)b.r + COVER_PAD;
     const int wxi = gb.x - ga.x, wyi = gb.y - ga.y, wzi = gb.z - ga.z;
     const long long R = b.r2 * ((long long)wxi * wxi + (long long)wyi * wyi + (long long)wzi * wzi);
-    q.e0 = make_int4(ga.x, ga.y, ga.z, wxi);
+    q.e0 = make_int4(ga.y * wzi - ga.z * wyi, ga.z * wxi - ga.x * wzi, ga.x * wyi - ga.y * wxi, wxi);
     q.e1 = make_int4(wyi, wzi, (int)(unsigned)(R & 0xffffffffll), (int)(R >> 32));
     const float ax = (float)ga.x, ay = (float)ga.y, az = (float)ga.z;
     const float wx = (float)wxi, wy = (float)wyi, wz = (float)wzi;
@@ -125,7 +125,7 @@ __device__ __forceinline__ int seed_setup(const Batch &b, int4 ga, int4 gb, int 
         }
     } else {                // second list: rows along y, index cy + ny * (cx + nx * cz)
         const int nx = b.ncy[0], ny = b.ncy[1], nz = b.ncy[2];
-        cs_off = (u32)view * (u32)b.ncelly;
+        cs_off = (u32)b.V * (u32)b.ncell + (u32)view * (u32)b.ncelly;
         ra = ay; rw = wy; rinv = b.icsy[1]; nr = ny;
         const int cx0 = max(0, floor_i(xl * b.icsy[0])), cx1 = min(nx - 1, floor_i(xh * b.icsy[0]));
         const int cz0 = max(0, floor_i(zl * b.icsy[2])), cz1 = min(nz - 1, floor_i(zh * b.icsy[2]));
@@ -142,7 +142,7 @@ __device__ __forceinline__ int seed_setup(const Batch &b, int4 ga, int4 gb, int 
     }
     const float3 os = slab_coeffs(oa, ow, oiw, ocs, pad);
     const float3 is = slab_coeffs(ia, iw, iiw, ics_, pad);
-    const int flags = (ylist ? 1 : 0) | (iw < 0.0f ? 2 : 0) | (rw < 0.0f ? 4 : 0);
+    const int flags = (iw < 0.0f ? 2 : 0) | (rw < 0.0f ? 4 : 0);
     q.e2 = make_float4(t0, t1, __int_as_float(o0), __int_as_float(0));
     q.e3 = make_float4(os.x, os.y, os.z, __int_as_float(nci));
     q.e4 = make_float4(is.x, is.y, is.z, iinv);
@@ -226,13 +226,12 @@ __device__ __forceinline__ void warp_items(const Batch &b, SeedTab &sp, int4 *tb
                 const float4 e4 = sp.f4(4, own), e5 = sp.f4(5, own), e6 = sp.f4(6, own);
                 const int4 e7 = sp.i4(7, own);
                 const int flags = __float_as_int(e5.w);
-                const int list = flags & 1;
                 const bool ineg = (flags & 2) != 0, rneg = (flags & 4) != 0;
                 // inner cells reached over [ta, tb]
                 const float il = fmaf(ineg ? tb : ta, e5.z, e5.x), ih = fmaf(ineg ? ta : tb, e5.z, e5.y);
                 const int nci = __float_as_int(e3.w);
                 const int ci0 = max(0, floor_i(il * e4.w)), ci1 = min(nci - 1, floor_i(ih * e4.w));
-                const u32 *__restrict__ cs = (list ? b.cell_start_y : b.cell_start) + (u32)e7.w;
+                const u32 *__restrict__ cs = b.cell_start + (u32)e7.w;
                 const int rowo = co * e7.y;
                 // cell run of inner cell ci: [s0, s1) into cs, or s0 = s1 = 0
                 auto run = [&](int ci, int &s0, int &s1) {
