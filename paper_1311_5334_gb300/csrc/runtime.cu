@@ -71,11 +71,15 @@ void *Ctx::take_stage(int kind, size_t bytes) {
             return p;
         }
     }
+    // relaxed: another thread may be capturing a stream, which the allocation leaves alone
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     void *p = nullptr;
     if (cudaHostAlloc(&p, bytes, cudaHostAllocPortable) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        p = nullptr;
     }
+    cudaThreadExchangeStreamCaptureMode(&mode);
     return p;
 }
 
@@ -88,7 +92,10 @@ void Ctx::give_stage(int kind, void *p) {
             return;
         }
     }
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     cudaFreeHost(p);
+    cudaThreadExchangeStreamCaptureMode(&mode);
 }
 
 Ctx::~Ctx() {
@@ -159,6 +166,8 @@ BatchRT::BatchRT(Ctx *c, const et_params &pp) : ctx(c), p(pp) {
 }
 
 BatchRT::~BatchRT() {
+    // the next owner of the stage must not see this batch's last run write it
+    if (done && cudaEventSynchronize(done) != cudaSuccess) cudaGetLastError();
     ctx->give_stage(0, stage);
     if (gexec) cudaGraphExecDestroy(gexec);
     if (done) cudaEventDestroy(done);
