@@ -49,12 +49,13 @@ OPS_PER_PAIR_TEST = 6
 # counts) moves, dram__bytes_read.sum + dram__bytes_write.sum of one ncu
 # capture of that launch (one pass, the first timed step, the kernel as built
 # now; profiles/k_tube_count_batched.md):
-#   batched  613.92 MB + 45.33 MB  (256 views, cells 74x621x506, both lists, 2 origins per ticket)
-# The kernel reads each view's grains and cell tables about once, so the bytes
-# follow the views and the cell shape rather than the seeds.  Keyed by
+#   batched  614.03 MB + 143.78 MB  (256 views, cells 74x621x506, both lists, 2 origins per ticket)
+# The kernel reads each view's grains and cell tables about once and writes its
+# candidates complete, so the bytes follow the views, the cell shape and the
+# candidates rather than the seeds.  Keyed by
 # (workload, views, cell edges, cell lists, origins per ticket); a run under
 # any other launch configuration reports null.
-TUBE_DRAM_BYTES = {("batched", 256, (74, 621, 506), 2, 2): 613.92e6 + 45.33e6}
+TUBE_DRAM_BYTES = {("batched", 256, (74, 621, 506), 2, 2): 614.03e6 + 143.78e6}
 
 
 def tube_run_key(workload, n_views, cell, tuning, rows=1, ticket_origins=0):
@@ -89,8 +90,8 @@ def measured_peaks():
         return {}
 # DRAM bytes of the front end's recognition kernel per view of raw frames
 # (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of 8 views:
-# 430.69 MB + 6.07 MB); a launch's traffic is scaled by its view count.
-FRAMES_DRAM_BYTES_PER_VIEW = (430.692608e6 + 6.068480e6) / 8
+# 441.1 MB + 7.3 MB); a launch's traffic is scaled by its view count.
+FRAMES_DRAM_BYTES_PER_VIEW = (441.1e6 + 7.3e6) / 8
 
 
 def dist_env():
