@@ -58,15 +58,17 @@ OPS_PER_PAIR_TEST = 6
 TUBE_DRAM_BYTES = {("batched", 256, (74, 621, 506), 2, 2): 614.03e6 + 143.78e6}
 
 
-def tube_run_key(workload, n_views, cell, tuning, rows=1, ticket_origins=0):
+def tube_run_key(workload, n_views, cell, tuning, rows=1, ticket_origins=0, grains=None):
     """Launch configuration of a tracking run, the key of TUBE_DRAM_BYTES:
     (workload, views, cell edges, cell lists, seed origins per ticket).
     tuning: the autotuner's choice, or None for edges fixed on the command
-    line (rows 1 = x rows only, else both lists; 0 origins = the default 2)."""
+    line (rows 1 = x rows only, else both lists; 0 origins = the automatic
+    size: 1 for a batch of at most 400,000 grains, else 2)."""
     if tuning is not None:
         lists, origins = int(tuning["row_lists"]), int(tuning["ticket_origins"])
     else:
-        lists, origins = (1 if rows == 1 else 2), (int(ticket_origins) or 2)
+        lists = 1 if rows == 1 else 2
+        origins = int(ticket_origins) or (1 if grains is not None and grains <= 400000 else 2)
     return (workload, int(n_views), tuple(int(c) for c in cell), lists, origins)
 
 
@@ -372,7 +374,7 @@ def run_ours(args):
     # configuration) over the same in-graph kernel time, against the measured
     # copy bandwidth: how far the kernel is from being bound by HBM
     run_key = tube_run_key(args.workload, n_views, ref_stats["cell"], batch.tuning if tuned else None,
-                           rows=args.rows, ticket_origins=args.ticket_origins)
+                           rows=args.rows, ticket_origins=args.ticket_origins, grains=ref_stats["n_grains"])
     traffic = TUBE_DRAM_BYTES.get(run_key)
     hbm = hbm_roofline(traffic, tube_avg_ms, measured_peaks())
 

@@ -214,6 +214,11 @@ void BatchRT::choose_cells() {
     ncelly = dual ? (long long)ncy[0] * ncy[1] * ncy[2] : 1;
 }
 
+// One origin per work ticket while a batch is small enough that the last
+// tickets' warps run alone (28k grains: tube counts 0.66 -> 0.60 ms); at 216k
+// grains one and two are equal, at 3.9 M two are 1.4 % faster.
+int BatchRT::auto_origins() const { return N <= 400000 ? 1 : 2; }
+
 // Autotuner: time the whole path for candidate cell shapes around the
 // density-based default s0 (about 0.35 grains per cell), each with one and
 // with both cell lists, then the seed generator's work-ticket size (origins
@@ -279,6 +284,7 @@ et_status BatchRT::autotune(cudaStream_t st, int max_trials, et_tuning *chosen, 
     if (saved.ticket_origins == 0) {   // origins per work ticket, for the fastest shape
         const et_tuning shape = best_t;
         for (int o : {1, 2, 4}) {
+            if (o == auto_origins()) continue;   // the shapes were timed with it
             et_tuning t = shape;
             t.ticket_origins = o;
             float ms = 0;
@@ -295,7 +301,7 @@ et_status BatchRT::autotune(cudaStream_t st, int max_trials, et_tuning *chosen, 
         }
     }
     profile = saved_prof;
-    if (best_t.ticket_origins == 0) best_t.ticket_origins = 2;   // the automatic choice, made explicit
+    if (best_t.ticket_origins == 0) best_t.ticket_origins = auto_origins();   // what was timed, made explicit
     tune = best_t;
     choose_cells();
     et_status s = reserve();
@@ -636,10 +642,7 @@ Batch BatchRT::dev_batch() const {
     b.r2 = (long long)p.tube_r * p.tube_r;
     b.flags = p.flags;
     b.spin_limit = tune.wait_polls > 0 ? (long long)tune.wait_polls : 0;
-    // one origin per work ticket while a batch is small enough that the last
-    // tickets' warps run alone (28k grains: tube counts 0.66 -> 0.60 ms); at 216k
-    // grains one and two are equal, at 3.9 M two are 1.4 % faster
-    b.gen_origins = tune.ticket_origins > 0 ? tune.ticket_origins : (N <= 400000 ? 1 : 2);
+    b.gen_origins = tune.ticket_origins > 0 ? tune.ticket_origins : auto_origins();
     const bool cut = (p.flags & ET_FLAG_ANGLE_CUT) != 0;
     b.cut_base = cut ? p.cut_base : 0;
     b.cut_slope = cut ? p.cut_slope : 0;

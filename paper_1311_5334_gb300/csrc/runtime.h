@@ -126,6 +126,7 @@ struct BatchRT {
     BatchRT(Ctx *c, const et_params &pp);
     ~BatchRT();
     void choose_cells();
+    int auto_origins() const;
     et_status autotune(cudaStream_t st, int max_trials, et_tuning *chosen, float *best_ms);
     void estimate_caps();
     size_t lay_group(int k, char *base, DevPtrs &P) const;
