@@ -321,7 +321,7 @@ def run_ours(args):
         cell, ms = batch.autotune(stream=stream)
         tuned = {"cell": list(cell), "row_lists": batch.tuning["row_lists"],
                  "ticket_origins": batch.tuning["ticket_origins"], "ms_per_run": ms,
-                 "how": "et_batch_autotune: fastest of 11 cell shapes, each with x rows and with x+y rows, "
+                 "how": "et_batch_autotune: fastest of 12 cell shapes, each with x rows and with x+y rows, "
                         "then 1, 2 or 4 seed origins per work ticket for that shape"}
 
     def step():

@@ -251,8 +251,9 @@ et_status et_batch_load(et_batch *b, const int32_t *xyz, const int64_t *offsets,
                         int32_t on_device, void *stream);
 et_status et_batch_set_tuning(et_batch *b, const et_tuning *tuning);
 /* Picks the tuning for the loaded batch by timing the whole path on it: up to
- * max_trials candidate cell shapes derived from the batch's mean grain
- * density (mostly anisotropic, cells along the x rows kept short), each with
+ * max_trials (0: all 12) cell shapes, the automatic one first and the others
+ * derived from the batch's mean grain density (mostly anisotropic, cells along
+ * the x rows kept short), each with
  * one cell list and with both lists, then 1, 2 and 4 origins per work ticket
  * for the fastest shape (unless ticket_origins was set); two runs each,
  * CUDA-event timed.  The fastest is kept as the batch's tuning and returned in

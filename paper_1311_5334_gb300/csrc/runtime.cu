@@ -219,10 +219,13 @@ void BatchRT::choose_cells() {
 // grains one and two are equal, at 3.9 M two are 1.4 % faster.
 int BatchRT::auto_origins() const { return N <= 400000 ? 1 : 2; }
 
-// Autotuner: time the whole path for candidate cell shapes around the
-// density-based default s0 (about 0.35 grains per cell), each with one and
-// with both cell lists, then the seed generator's work-ticket size (origins
-// per ticket) for the fastest shape, and keep the fastest combination.
+// Autotuner: time the whole path for the automatic cell shape and for
+// candidate shapes around the edge s0 of a cube holding 0.35 grains at the
+// batch's mean density, each with one and with both cell lists, then the seed
+// generator's work-ticket size (origins per ticket) for the fastest shape, and
+// keep the fastest combination.  The two scales differ where views do (1.2 on
+// 256 lognormal views, where s0 (0.16, 1.35, 1.1) is the fastest: 67.5 ms
+// against 67.7 for the automatic shape).
 et_status BatchRT::autotune(cudaStream_t st, int max_trials, et_tuning *chosen, float *best_ms) {
     if (!loaded) return fail(ET_ERR_NOT_READY, "no grains loaded");
     if (!st) st = ctx->stream;
@@ -233,9 +236,12 @@ et_status BatchRT::autotune(cudaStream_t st, int max_trials, et_tuning *chosen, 
     static const double cand[][3] = {{0.22, 1.1, 1.1}, {0.33, 1.3, 1.3}, {0.16, 1.1, 1.1}, {0.27, 0.95, 0.95},
                                      {0.22, 1.3, 1.3}, {0.33, 1.1, 1.1}, {0.5, 1.6, 1.3}, {1.0, 1.0, 1.0},
                                      {0.16, 1.22, 1.22}, {0.16, 1.35, 1.1}, {0.18, 1.6, 1.6}};
-    const int ncand = (int)(sizeof cand / sizeof cand[0]);
+    const int ncand = 1 + (int)(sizeof cand / sizeof cand[0]);   // the automatic shape is the first
     if (max_trials <= 0 || max_trials > ncand) max_trials = ncand;
     const et_tuning saved = tune;
+    for (int a = 0; a < 3; ++a) tune.cell[a] = 0;
+    choose_cells();
+    const int auto_cs[3] = {cs[0], cs[1], cs[2]};
     const bool saved_prof = profile;
     profile = true;
     float best = 3.0e38f;
@@ -267,7 +273,8 @@ et_status BatchRT::autotune(cudaStream_t st, int max_trials, et_tuning *chosen, 
     for (int k = 0; k < 2 * max_trials; ++k) {   // every shape with one and with both cell lists
         et_tuning t = saved;
         for (int a = 0; a < 3; ++a)
-            t.cell[a] = std::max(16, std::min(p.extent[a], (int)std::lround(s0 * cand[k / 2][a])));
+            t.cell[a] = k < 2 ? auto_cs[a]
+                              : std::max(16, std::min(p.extent[a], (int)std::lround(s0 * cand[k / 2 - 1][a])));
         t.row_lists = 1 + (k & 1);
         float ms = 0;
         et_status s = trial(t, ms);

@@ -21,3 +21,20 @@ def test_kept_ticket_size_was_timed():
             b.autotune(max_trials=1)
             kept.append(b.tuning["ticket_origins"])
     assert kept == [1] * 8
+
+
+@pytest.mark.parametrize("views", [1, 3])
+def test_automatic_cells_are_the_first_trial(views):
+    """With one shape to try, the cells kept are those an untuned batch uses."""
+    import numpy as np
+    from paper_1311_5334_gb300 import et
+
+    vs = [synth.make_view([8, k], n_fog=(6000, 400, 300)[k], n_through=10) for k in range(views)]
+    offs = np.concatenate([[0], np.cumsum([v.n for v in vs])])
+    with et.Context(0) as ctx, et.Batch(ctx, synth.params(vs[0].extent)) as b:
+        b.load(np.concatenate([v.xyz for v in vs]), offs)
+        b.find()
+        b.fetch()
+        automatic = b.stats()["cell"]
+        cell, _ = b.autotune(max_trials=1)
+    assert cell == automatic
