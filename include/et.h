@@ -112,9 +112,11 @@ typedef struct {
 typedef struct {
     int32_t cell[3];        /* cell-list edge per axis, coordinate units; 0: automatic
                                (s0 * (0.24, 1.9, 1.5), s0 the edge of a cube holding 0.35
-                               grains at the density the work sees).  The batch's cell table
-                               (views x cells per view) must stay below 2^31 - 1 cells, else
-                               loading fails with ET_ERR_INVALID_ARG */
+                               grains at the density the work sees; larger where the cells
+                               of a batch of unlike views would pass 2^28, or where memory is
+                               short).  Each cell list of the batch (views x cells per view)
+                               must stay below 2^31 - 1 cells, else loading fails with
+                               ET_ERR_INVALID_ARG */
     int32_t ticket_origins; /* origins per work ticket of the seed generator (a warp takes
                                this many consecutive grains as line origins at a time):
                                1, 2 or 4; 0: automatic (1 up to 400,000 grains in

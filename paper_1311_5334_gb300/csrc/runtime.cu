@@ -181,24 +181,16 @@ BatchRT::~BatchRT() {
 // it with 32-bit signed arithmetic.
 static constexpr double kMaxCells = 2147483647.0;
 
-void BatchRT::choose_cells() {
-    for (int k = 0; k < 3; ++k) cs[k] = tune.cell[k];
-    if (cs[0] <= 0 || cs[1] <= 0 || cs[2] <= 0) {
-        // s0: the edge of a cube holding 0.35 grains at the density the work sees (a
-        // view's tube tests grow with the cube of its grains: seeds times grains
-        // along a line).  Cells are short along the x rows and long across them.
-        // Sweeps of 13 shapes on views of 2.5k to 65k grains, a 1.2 M-grain scan and
-        // batches of 17 and 256 views put this shape, or one within 2 % of it, first;
-        // against 0.22, 1.1, 1.1 at the batch's mean density the 28k view's tube
-        // counts took 0.66 instead of 0.72 ms and the scan 203 instead of 321 ms
-        double vol = (double)p.extent[0] * p.extent[1] * p.extent[2];
-        double nwork = sum_n2 > 0.0 ? sum_n3 / sum_n2 : 1.0;
-        double rho = std::max(nwork, 1.0) / vol;
-        double s = std::cbrt(0.35 / rho);
-        s = std::min(std::max(s, 64.0), 4096.0);
-        for (int k = 0; k < 3; ++k)
-            if (tune.cell[k] <= 0) cs[k] = std::max(16, (int)std::lround(s * AUTO_CELL[k]));
-    }
+// Cells of the automatic table, both lists together, above which a batch of unlike
+// views gets larger cells than its dense views would choose, down to the number
+// the mean density gives.  One view of 60k grains among small ones, ms a call at
+// limits of 2^26 / 2^27 / 2^28 cells, and without: among 1,000 6.6 / 5.5 / 4.9 / 5.5,
+// among 4,000 12.9 / 10.4 / 7.2 / 10.8, among 10,000 20.3 / 17.0 / 10.9 (without, the
+// table is beyond its limit).
+static constexpr double kRoomyCells = (double)(1ll << 28);
+
+// The cell grids of the edges cs.
+void BatchRT::lay_grid() {
     for (int k = 0; k < 3; ++k) {
         cs[k] = std::max(1, std::min(cs[k], p.extent[k]));
         nc[k] = (p.extent[k] + cs[k] - 1) / cs[k];
@@ -212,6 +204,33 @@ void BatchRT::choose_cells() {
     csy[2] = cs[2];
     for (int k = 0; k < 3; ++k) ncy[k] = (p.extent[k] + csy[k] - 1) / csy[k];
     ncelly = dual ? (long long)ncy[0] * ncy[1] * ncy[2] : 1;
+}
+
+void BatchRT::choose_cells() {
+    for (int k = 0; k < 3; ++k) cs[k] = tune.cell[k];
+    if (cs[0] > 0 && cs[1] > 0 && cs[2] > 0) return lay_grid();
+    const double vol = (double)p.extent[0] * p.extent[1] * p.extent[2];
+    // s0: the edge of a cube holding 0.35 of a view's grains
+    auto edge = [&](double grains) { return std::min(std::max(std::cbrt(0.35 * vol / std::max(grains, 1.0)), 64.0), 4096.0); };
+    // lays the grids of the edges s f where none is set; returns the table's cells
+    auto lay = [&](double s, const double *f) {
+        for (int k = 0; k < 3; ++k) cs[k] = tune.cell[k] > 0 ? tune.cell[k] : std::max(16, (int)std::lround(s * f[k]));
+        lay_grid();
+        return (double)V * (double)(ncell + (dual ? ncelly : 0));
+    };
+    // s0 at the density the work sees (a view's tube tests grow with the cube of
+    // its grains: seeds times grains along a line).  Cells are short along the x
+    // rows and long across them.  Sweeps of 13 shapes on views of 2.5k to 65k
+    // grains, a 1.2 M-grain scan and batches of 17 and 256 views put this shape, or
+    // one within 2 % of it, first; against 0.22, 1.1, 1.1 at the batch's mean
+    // density the 28k view's tube counts took 0.66 instead of 0.72 ms and the scan
+    // 203 instead of 321 ms
+    double s = edge(sum_n2 > 0.0 ? sum_n3 / sum_n2 : 1.0);
+    const double room = tight_cells ? 0.0 : kRoomyCells;
+    if (lay(s, AUTO_CELL) <= room) return;
+    static const double mean_shape[3] = {0.22, 1.1, 1.1};
+    const double limit = std::max(room, lay(edge(V > 0 ? (double)N / V : 1.0), mean_shape));
+    while (lay(s, AUTO_CELL) > limit) s *= 1.1;   // ends: one cell a view is within the limit
 }
 
 // One origin per work ticket while a batch is small enough that the last
@@ -609,12 +628,18 @@ et_status BatchRT::load(const int32_t *xyz, const int64_t *offsets, int nv, bool
         sum_n3 += k * k * k;
     }
     for (int k = 0; k < 3; ++k) cbits[k] = cb[k];
+    tight_cells = false;
     choose_cells();
     if ((double)V * (double)std::max(ncell, ncelly) >= kMaxCells)
         return fail(ET_ERR_INVALID_ARG, "cell table of %.3g cells too large (limit 2^31 - 1)",
                     (double)V * (double)std::max(ncell, ncelly));
     estimate_caps();
     et_status s = reserve();
+    if (s == ET_ERR_OOM) {   // again with the smallest automatic cell table
+        tight_cells = true;
+        choose_cells();
+        s = reserve();
+    }
     if (s != ET_OK) return s;
     if (!stage) stage = (Stage *)ctx->take_stage(0, sizeof(Stage));
     cudaError_t e = cudaMemcpyAsync(goff, goff_h.data(), sizeof(long long) * (V + 1), cudaMemcpyHostToDevice, st);

@@ -75,6 +75,7 @@ struct BatchRT {
     int csy[3] = {1, 1, 1}, ncy[3] = {1, 1, 1};   // second cell list (rows along y)
     long long ncelly = 1;
     bool dual = false;
+    bool tight_cells = false;   // memory is short: the automatic cell table takes no more than the mean density's
     // requested capacities
     u64 want_cand = 0, want_members = 0, want_rec = 0;
     // granted capacities
@@ -125,6 +126,7 @@ struct BatchRT {
 
     BatchRT(Ctx *c, const et_params &pp);
     ~BatchRT();
+    void lay_grid();
     void choose_cells();
     int auto_origins() const;
     et_status autotune(cudaStream_t st, int max_trials, et_tuning *chosen, float *best_ms);
