@@ -617,6 +617,7 @@ et_status BatchRT::load(const int32_t *xyz, const int64_t *offsets, int nv, bool
     for (int k = 0; k < 3; ++k) cb[k] = bits_for((unsigned long long)(p.extent[k] - 1));
     int vb = bits_for((unsigned long long)std::max(nv - 1, 0));
     if (cb[0] + cb[1] + cb[2] + vb > 64) return fail(ET_ERR_INVALID_ARG, "too many views for the key width");
+    loaded = ran = false;   // from here on the shape is the new one: a load that fails leaves nothing to find or fetch
     V = nv;
     N = total;
     maxN = mx;
@@ -648,7 +649,6 @@ et_status BatchRT::load(const int32_t *xyz, const int64_t *offsets, int nv, bool
                             on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail(e, "grain upload");
     loaded = true;
-    ran = false;
     return ET_OK;
 }
 
