@@ -289,6 +289,15 @@ et_status BatchRT::autotune(cudaStream_t st, int max_trials, et_tuning *chosen, 
         ms_out = t_best;
         return ET_OK;
     };
+    // back to the tuning before; the buffers are laid out for it by the next find
+    auto give_up = [&](et_status s) {
+        if (cudaStreamSynchronize(st) != cudaSuccess) cudaGetLastError();
+        tune = saved;
+        profile = saved_prof;
+        choose_cells();
+        laid = ran = false;
+        return s;
+    };
     for (int k = 0; k < 2 * max_trials; ++k) {   // every shape with one and with both cell lists
         et_tuning t = saved;
         for (int a = 0; a < 3; ++a)
@@ -297,11 +306,7 @@ et_status BatchRT::autotune(cudaStream_t st, int max_trials, et_tuning *chosen, 
         t.row_lists = 1 + (k & 1);
         float ms = 0;
         et_status s = trial(t, ms);
-        if (s != ET_OK) {
-            tune = saved;
-            profile = saved_prof;
-            return s;
-        }
+        if (s != ET_OK) return give_up(s);
         if (ms >= 0.0f && ms < best) {
             best = ms;
             best_t = t;
@@ -315,11 +320,7 @@ et_status BatchRT::autotune(cudaStream_t st, int max_trials, et_tuning *chosen, 
             t.ticket_origins = o;
             float ms = 0;
             et_status s = trial(t, ms);
-            if (s != ET_OK) {
-                tune = saved;
-                profile = saved_prof;
-                return s;
-            }
+            if (s != ET_OK) return give_up(s);
             if (ms >= 0.0f && ms < best) {
                 best = ms;
                 best_t = t;
@@ -488,6 +489,7 @@ void BatchRT::release_groups() {
 }
 
 et_status BatchRT::reserve() {
+    laid = false;   // a group given back and not had again leaves its arrays' pointers behind
     size_t sizes[NGROUP];
     plan_groups(sizes);
     if (byte_limit && footprint_with(sizes) > byte_limit)
@@ -546,6 +548,7 @@ et_status BatchRT::reserve() {
         cap_rec = want_rec;
     }
     temp = g_temp.base;
+    laid = true;
     return ET_OK;
 }
 
@@ -805,6 +808,7 @@ et_status BatchRT::find(cudaStream_t st, bool use_graph) {
     if (!loaded) return fail(ET_ERR_NOT_READY, "no grains loaded");
     if (!st) st = ctx->stream;
     et_status s;
+    if (!laid && (s = reserve()) != ET_OK) return s;   // an earlier call ran out of memory
     if (use_graph && N > 0) {
         const unsigned long long key = graph_signature() ^ (profile ? 0x8000000000000000ull : 0ull);
         if (!gexec || key != graph_key) {
@@ -951,7 +955,7 @@ void BatchRT::mark(int stage, cudaStream_t st) {
 int BatchRT::count_kernels() {
     const unsigned long long key = graph_signature();
     if (kernel_launches >= 0 && key == launches_key) return kernel_launches;
-    if (!loaded || N == 0) return 0;
+    if (!loaded || !laid || N == 0) return 0;
     cudaStream_t st = nullptr;
     if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) return -1;
     const bool prof = profile;

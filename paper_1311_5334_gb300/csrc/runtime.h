@@ -112,6 +112,7 @@ struct BatchRT {
     cudaEvent_t done = nullptr;
     cudaStream_t run_stream = nullptr;
     bool loaded = false, ran = false;
+    bool laid = false;        // the arrays' pointers are those of the groups held
     bool full_sort = false;   // the canonical order sorts all key bits (grains crowd on shared x)
     Ctl hctl{};
     Stage *stage = nullptr;   // null: results are copied by the fetch

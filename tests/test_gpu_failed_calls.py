@@ -41,3 +41,72 @@ def test_failed_load_leaves_nothing_to_fetch(oracle_mod):
                 with pytest.raises(et.EtError) as e:
                     call()
                 assert e.value.status == et.NOT_READY
+
+
+class Memory:
+    """Allocation hooks through PyTorch's allocator that can be told to refuse."""
+
+    def __init__(self, et, ctx):
+        import torch
+
+        self.refuse = False
+
+        def alloc(nbytes, _):
+            return None if self.refuse else torch.cuda.caching_allocator_alloc(int(nbytes), 0)
+
+        self.hooks = (et.ALLOC_FN(alloc), et.FREE_FN(lambda ptr, _: torch.cuda.caching_allocator_delete(ptr)))
+        et._check(et.lib().et_ctx_set_allocator(ctx._h, self.hooks[0], self.hooks[1], None))
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_run_after_growing_the_buffers_failed(oracle_mod, graph):
+    """More candidates than the first buffers hold, and no memory for larger ones: neither a fetch nor another
+    run uses buffers that were given back."""
+    pytest.importorskip("torch")
+    from paper_1311_5334_gb300 import et
+
+    v = synth.make_view(51, n_fog=6000, n_through=40)
+    p = synth.params(v.extent, min_hits=2)
+    want = want_of(oracle_mod, v.xyz, p)
+    with et.Context(0) as ctx:
+        mem = Memory(et, ctx)
+        with et.Batch(ctx, p) as b:
+            b.load(v.xyz, [0, v.n])
+            mem.refuse = True
+            b.find(use_graph=graph)
+            for call in (b.fetch, b.fetch, lambda: b.find(use_graph=graph), lambda: b.find(use_graph=graph)):
+                with pytest.raises(et.EtError) as e:
+                    call()
+                assert e.value.status == et.OOM
+            mem.refuse = False
+            b.find(use_graph=graph)
+            tracks, members, _ = b.fetch()
+            assert b.stats()["n_candidates"] > 65536
+    assert et.track_tuples(tracks, members) == want
+
+
+def test_run_after_a_failed_autotune(oracle_mod):
+    """No memory for a trial's cell table: the tuning of before is kept and laid out again."""
+    pytest.importorskip("torch")
+    from paper_1311_5334_gb300 import et
+
+    v = synth.make_view(52, n_fog=3000, n_through=30)
+    p = synth.params(v.extent)
+    want = want_of(oracle_mod, v.xyz, p)
+    with et.Context(0) as ctx:
+        mem = Memory(et, ctx)
+        with et.Batch(ctx, p) as b:
+            b.set_tuning(cell=(2000, 4000, 4000), row_lists=1)   # a table smaller than any trial's
+            b.load(v.xyz, [0, v.n])
+            mem.refuse = True
+            with pytest.raises(et.EtError) as e:
+                b.autotune()
+            assert e.value.status == et.OOM
+            with pytest.raises(et.EtError) as e:
+                b.find()
+            assert e.value.status == et.OOM
+            mem.refuse = False
+            b.find()
+            tracks, members, _ = b.fetch()
+            assert b.stats()["cell"] == (2000, 4000, 4000)
+    assert et.track_tuples(tracks, members) == want
