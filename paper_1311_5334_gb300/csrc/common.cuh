@@ -54,7 +54,8 @@ struct Ctl {
     u64 ncl[2];         // merge: lengths of the undecided-candidate lists (ping-pong)
     u32 round_active[64];   // merge: participants of the first 64 rounds (diagnostics)
     u64 ticket[2];          // work tickets of the tube-count and member-list kernels
-    u32 n_long, pad2;       // tracks in Out::long_tracks
+    u32 n_long;             // tracks in Out::long_tracks
+    u32 crowded;            // the full sort found grains that crowd on shared x
     u64 n_pair_tests;       // seed-window tests of the seed generator
 };
 
@@ -284,9 +285,10 @@ void exclusive_scan_u64_dev(const u64 *in, u64 *out, long long n_cap, const u64 
 
 // grid.cu
 void launch_canonical_keys(const Batch &b, u64 *keys, u32 *vals, cudaStream_t st);
-// keys: in order of their bits from bit0 on
+// keys: in order of their bits from bit0 on; with bit0 = 0 and watch > 0, grains that
+// would crowd with bit0 = watch set Ctl::crowded
 void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y, int bit0,
-                            cudaStream_t st);
+                            int watch, cudaStream_t st);
 // cursors: the cell starts, which the scatter counts up
 void launch_cell_scatter(const Batch &b, u32 *cursor, u32 *cursor_y, cudaStream_t st);
 

@@ -55,10 +55,12 @@ __device__ __forceinline__ u32 cell_y(const Batch &b, int v, int x, int y, int z
 // that agree there, rarely more than one, comes from comparing the full keys.
 // Sorting on all bits took 6 instead of 2 passes for one view.  More than
 // CROWD grains that agree report ERRB_CROWDED, and the run is repeated with
-// the full sort.
+// the full sort, as are the batch's next ones; those watch whether grains would
+// still crowd.
 constexpr int CROWD = 64;
 
-__global__ void k_canonical_order(Batch b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y, int bit0) {
+__global__ void k_canonical_order(Batch b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y, int bit0,
+                                  int watch) {
     griddep_launch();
     griddep_wait();
     // a coordinate out of range is reported as such; a timed-out sort leaves
@@ -84,6 +86,7 @@ __global__ void k_canonical_order(Batch b, const u64 *keys, const u32 *vals, u32
             }
         } else {
             twin = q > b.goff[v] && keys[q - 1] == key;
+            if (watch && q + CROWD + 1 < b.N && (keys[q + CROWD + 1] >> watch) == (key >> watch)) b.ctl->crowded = 1;
         }
         if (crowded) {
             atomicOr(&b.ctl->error, ERRB_CROWDED);
@@ -135,8 +138,8 @@ void launch_canonical_keys(const Batch &b, u64 *keys, u32 *vals, cudaStream_t st
 }
 
 void launch_canonical_order(const Batch &b, const u64 *keys, const u32 *vals, u32 *count, u32 *count_y, int bit0,
-                            cudaStream_t st) {
-    launch_dep(k_canonical_order, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, keys, vals, count, count_y, bit0);
+                            int watch, cudaStream_t st) {
+    launch_dep(k_canonical_order, dim3(grid_for(b.N, 256)), dim3(256), 0, st, b, keys, vals, count, count_y, bit0, watch);
 }
 
 void launch_cell_scatter(const Batch &b, u32 *cursor, u32 *cursor_y, cudaStream_t st) {

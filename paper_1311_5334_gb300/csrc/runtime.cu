@@ -597,7 +597,7 @@ unsigned long long BatchRT::graph_signature() const {
     mix((unsigned long long)tune.wait_polls);
     mix((unsigned long long)tune.ticket_origins);
     mix((unsigned long long)tune.assoc_window);
-    mix(full_sort ? 1ull : 0ull);
+    mix(crowd_loads > 0 ? 1ull : 0ull);
     mix((unsigned long long)(uintptr_t)stage);
     return h;
 }
@@ -620,6 +620,7 @@ et_status BatchRT::load(const int32_t *xyz, const int64_t *offsets, int nv, bool
     for (int k = 0; k < 3; ++k) cb[k] = bits_for((unsigned long long)(p.extent[k] - 1));
     int vb = bits_for((unsigned long long)std::max(nv - 1, 0));
     if (cb[0] + cb[1] + cb[2] + vb > 64) return fail(ET_ERR_INVALID_ARG, "too many views for the key width");
+    if (crowd_loads > 0) --crowd_loads;
     loaded = ran = false;   // from here on the shape is the new one: a load that fails leaves nothing to find or fetch
     V = nv;
     N = total;
@@ -765,10 +766,10 @@ et_status BatchRT::enqueue(cudaStream_t st, bool record) {
         launch_canonical_keys(b, keys[0], vals[0], st);
         const int kb = b.vshift + bits_for((unsigned long long)std::max(V - 1, 0));
         // on view and x alone while few grains of a view can share their x
-        const int bit0 = !full_sort && maxN <= 4 * (long long)p.extent[0] ? cbits[1] + cbits[2] : 0;
+        const int xbit = maxN <= 4 * (long long)p.extent[0] ? cbits[1] + cbits[2] : 0, bit0 = crowd_loads > 0 ? 0 : xbit;
         int c1 = radix_sort_pairs(keys[0], vals[0], keys[1], vals[1], n, kb - bit0, temp, st, &ctl->error, ERRB_TIMEOUT,
                                   ctl->bar, b.spin_limit, bit0);
-        launch_canonical_order(b, keys[c1], vals[c1], cell_count, cell_count + cells, bit0, st);
+        launch_canonical_order(b, keys[c1], vals[c1], cell_count, cell_count + cells, bit0, bit0 ? 0 : xbit, st);
         // both cell lists by one counting sort: the scan leaves the starts, and in
         // the counts' place a copy that serves as the scatter's cursors
         exclusive_scan_u32(cell_count, cell_start, (long long)(cells + cellsy), temp, st, &ctl->error, ERRB_TIMEOUT,
@@ -866,6 +867,7 @@ et_status BatchRT::settle(bool record) {
         if (hctl.error & ERRB_OUT_OF_RANGE) return fail(ET_ERR_OUT_OF_RANGE, "a grain lies outside [0, extent)");
         if (hctl.error & ERRB_DUPLICATE) return fail(ET_ERR_DUPLICATE_GRAIN, "two grains share coordinates");
         if (hctl.error & ERRB_TIMEOUT) return fail(ET_ERR_TIMEOUT, "device-side wait timed out (merge barrier or sort look-back)");
+        if ((hctl.error & ERRB_CROWDED) || hctl.crowded) crowd_loads = CROWD_LOADS;
         if (!(hctl.error & ERRB_OVF_MASK)) return ET_OK;
         if (attempt >= 6) return fail(ET_ERR_CAPACITY, "internal buffers kept overflowing");
         if (hctl.error & ERRB_OVF_CAND) {
@@ -873,7 +875,6 @@ et_status BatchRT::settle(bool record) {
             want_members = std::max<u64>(want_members, want_cand * 24);
         }
         if (hctl.error & ERRB_OVF_MEMBERS) want_members = std::max<u64>(want_members, hctl.n_members + 1024);
-        if (hctl.error & ERRB_CROWDED) full_sort = true;
         if (hctl.error & ERRB_OVF_RECORD) want_rec = std::max<u64>(want_rec, hctl.n_seeds);
         s = reserve();
         if (s != ET_OK) return s;

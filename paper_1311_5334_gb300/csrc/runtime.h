@@ -113,7 +113,10 @@ struct BatchRT {
     cudaStream_t run_stream = nullptr;
     bool loaded = false, ran = false;
     bool laid = false;        // the arrays' pointers are those of the groups held
-    bool full_sort = false;   // the canonical order sorts all key bits (grains crowd on shared x)
+    // loads, this one included, whose canonical order sorts all key bits: grains crowd
+    // on shared x, now or a few loads ago (a stream that alternates is not run twice)
+    int crowd_loads = 0;
+    static constexpr int CROWD_LOADS = 8;
     Ctl hctl{};
     Stage *stage = nullptr;   // null: results are copied by the fetch
     cudaGraphExec_t gexec = nullptr;
