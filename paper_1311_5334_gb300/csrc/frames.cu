@@ -422,6 +422,7 @@ struct FramesRT {
             view_off = cv.take<u32>((size_t)V + 1);
             temp = cv.take<char>(scan_temp_bytes((long long)rows()));
         };
+        cap = last_views = 0;   // until the arrays are there
         carve(c);
         if (!g_out.reserve(ctx, c.off)) return fail(ET_ERR_OOM, "grain buffers (%llu grains)", (unsigned long long)need);
         Carver d;
@@ -486,6 +487,7 @@ struct FramesRT {
         if (ran) cudaEventSynchronize(ev[3]);
         if (handoff_pending) cudaEventSynchronize(handoff);   // buffers may be regrown below
         handoff_pending = false;
+        ran = false;   // the shape is the new one: a run that fails leaves nothing to fetch
         V = nv;
         const size_t bytes = (size_t)nv * view_bytes();
         cudaEventRecord(ev[0], st);
@@ -497,14 +499,21 @@ struct FramesRT {
             if (e != cudaSuccess) return cuda_fail(e, "raw frame upload");
             d_raw = (const unsigned char *)g_raw.base;
         }
-        want = std::max(want, std::max<u64>(65536, (u64)nv * p.depth * p.height * p.width / 2000));
-        if (cap < want || (size_t)V > last_views) {
-            et_status s = reserve_out(std::max(want, cap));
-            if (s != ET_OK) return s;
+        const u64 need = std::max(want, std::max<u64>(65536, (u64)nv * p.depth * p.height * p.width / 2000));
+        if (cap < need || (size_t)V > last_views) {
+            et_status s = reserve_out(std::max(need, cap));
+            if (s != ET_OK) {
+                if (!on_device) cudaStreamSynchronize(st);   // the upload
+                return s;
+            }
         }
+        want = need;
         et_status s = enqueue(st);
-        if (s != ET_OK) return s;
         cudaEventRecord(ev[3], st);
+        if (s != ET_OK) {
+            cudaEventSynchronize(ev[3]);   // what was launched still writes this handle's memory
+            return s;
+        }
         run_stream = st;
         ran = true;
         settled = false;
@@ -532,9 +541,10 @@ struct FramesRT {
                 settled = true;
                 return run_status = ET_OK;
             }
-            want = hctl.n_grains + hctl.n_grains / 8 + 1024;
-            et_status s = reserve_out(want);
+            const u64 need = hctl.n_grains + hctl.n_grains / 8 + 1024;
+            et_status s = reserve_out(need);
             if (s != ET_OK) return run_status = s;
+            want = need;
             cudaStream_t st = ctx->stream;
             cudaEventRecord(ev[0], st);
             s = enqueue(st);

@@ -110,3 +110,74 @@ def test_run_after_a_failed_autotune(oracle_mod):
             tracks, members, _ = b.fetch()
             assert b.stats()["cell"] == (2000, 4000, 4000)
     assert et.track_tuples(tracks, members) == want
+
+
+def stack(seed):
+    return synth.random_blobs((5, 40, 64), n=30, seed=seed)
+
+
+def frames_of(et, ctx, f):
+    d, h, pitch = f.raw.shape
+    fp = et.make_frame_params(f.width, h, d, synth.PITCH_NUM, synth.PITCH_DEN, synth.GRAIN_THRESHOLD, row_pitch=pitch)
+    return et.Frames(ctx, fp, f.gain, f.thr)
+
+
+def frames_want(oracle_mod, f):
+    g = oracle_mod.frames_filter(f.raw, f.gain, f.thr)
+    return oracle_mod.frames_grains(g, synth.GRAIN_THRESHOLD, synth.PITCH_NUM, synth.PITCH_DEN)
+
+
+def test_failed_frames_run_leaves_nothing_to_fetch(oracle_mod):
+    """No memory for the upload of three stacks after a run of one."""
+    pytest.importorskip("torch")
+    from paper_1311_5334_gb300 import et
+
+    f = stack(81)
+    wx, wp, _ = frames_want(oracle_mod, f)
+    with et.Context(0) as ctx:
+        mem = Memory(et, ctx)
+        with frames_of(et, ctx, f) as fr, et.Batch(ctx, synth.params(synth.FRAME_EXTENT)) as b:
+            for _ in range(2):
+                fr.run(f.raw, n_views=1)
+                xyz, pulse, voff = fr.fetch()
+                assert np.array_equal(xyz, wx) and np.array_equal(pulse, wp) and list(voff) == [0, len(wx)]
+                mem.refuse = True
+                with pytest.raises(et.EtError) as e:
+                    fr.run(np.tile(f.raw.reshape(-1), 3), n_views=3)
+                assert e.value.status == et.OOM
+                for call in (fr.fetch, lambda: fr.to_batch(b)):
+                    with pytest.raises(et.EtError) as e:
+                        call()
+                    assert e.value.status == et.NOT_READY
+                mem.refuse = False
+
+
+def test_frames_run_after_failed_grain_buffers(oracle_mod):
+    """Rows of 40 stacks need larger buffers than those of one, and there is no memory: the next runs, larger or
+    smaller, use no buffers that were given back."""
+    torch = pytest.importorskip("torch")
+    from paper_1311_5334_gb300 import et
+
+    f = stack(82)
+    wx, wp, _ = frames_want(oracle_mod, f)
+    one = torch.from_numpy(f.raw.reshape(-1).copy()).cuda()
+    many = one.repeat(40)
+    with et.Context(0) as ctx:
+        mem = Memory(et, ctx)
+        with frames_of(et, ctx, f) as fr:
+            fr.run(one, n_views=1)
+            fr.fetch()
+            mem.refuse = True
+            for raw, n in ((many, 40), (one, 1), (many, 40), (one, 1)):
+                with pytest.raises(et.EtError) as e:
+                    fr.run(raw, n_views=n)
+                assert e.value.status == et.OOM
+                with pytest.raises(et.EtError) as e:
+                    fr.fetch()
+                assert e.value.status == et.NOT_READY
+            mem.refuse = False
+            for raw, n in ((one, 1), (many, 40)):
+                fr.run(raw, n_views=n)
+                xyz, pulse, voff = fr.fetch()
+                assert np.array_equal(xyz, np.tile(wx, (n, 1))) and np.array_equal(pulse, np.tile(wp, n))
+                assert list(voff) == [k * len(wx) for k in range(n + 1)]
