@@ -60,7 +60,9 @@ typedef struct {
     int64_t n_grains;
     float kernel_ms;         /* CUDA-event time of the recognition kernel (filtering and grains) */
     float run_ms;            /* CUDA-event time of the whole run on the device (upload included) */
-    int32_t kernel_launches; /* kernels one run launches (recognition, scan of the row counts, placement) */
+    int32_t kernel_launches; /* kernels the run launched: recognition, scan of the row counts, placement and
+                                publication; three more where image rows are crowded (over 384 grains, or over
+                                64 in a run of more than 2^19) */
     int32_t reserved;
 } et_frames_stats;
 

@@ -42,7 +42,7 @@ constexpr int FT = 256;       // threads per block
 constexpr int ZC = 8;         // frames a scanning thread holds at a time
 constexpr int QCAP = 16 * FT; // candidates a block collects on chip: at least one frame of its tile
 
-enum : u32 { FRB_OVF = 1u << 0, FRB_TIMEOUT = 1u << 1 };
+enum : u32 { FRB_OVF = 1u << 0, FRB_TIMEOUT = 1u << 1, FRB_CROWDED = 1u << 2 };
 
 struct FrCtl {
     u64 n_grains;   // grains appended (may exceed the capacity)
@@ -285,19 +285,66 @@ __global__ void __launch_bounds__(FT, 4) k_recognize(const __grid_constant__ FrA
 }
 
 // Grains into raster order: a grain's place is its row's start plus its rank by
-// x among the row's grains (a few).  Also the views' offsets.
+// x among the row's grains (a few).  Also the views' offsets.  Every grain of a
+// row walks its whole chain, so longer rows are left to the two kernels below,
+// which the host then launches.  us a call by chains and by those kernels: rows of
+// 256 grains 65 and 75 (one row), 150 and 153 (66k grains); of 320, 150 and 153
+// (82k grains); of 512, 83 and 85 (one row), 312 and 283 (262k grains); of 1,024,
+// 199 and 138 (16k grains).  Above ROW_FEW grains the kernels win from rows of some
+// 65 on: 933k grains of noise, 114 a row, 1,344 and 980; 4.2 M grains, 2,048 a row,
+// 9,582 and 6,787.
+constexpr u32 ROW_WALK = 384, ROW_WALK_LARGE = 64, ROW_FEW = 1u << 19;
+
 __global__ void k_fr_place(FrArgs a, const u32 *row_start, int *xyz, int *pulse, u32 *view_off) {
     griddep_launch();
     griddep_wait();
     const u64 n = min(a.ctl->n_grains, a.cap);
+    const u32 limit = n > ROW_FEW ? ROW_WALK_LARGE : ROW_WALK;
     const u64 tid = (u64)blockIdx.x * blockDim.x + threadIdx.x, stride = (u64)gridDim.x * blockDim.x;
     for (u64 v = tid; v <= (u64)a.V; v += stride) view_off[v] = row_start[v * (u64)a.D * a.H];
     for (u64 i = tid; i < n; i += stride) {
         const u64 k = a.key[i], row = k >> 12;
+        const u32 r0 = row_start[row];
+        if (row_start[row + 1] - r0 > limit) {
+            atomicOr(&a.ctl->error, FRB_CROWDED);
+            continue;
+        }
         u32 rank = 0;
         for (u32 j = a.row_head[row]; j != ~0u; j = a.next[j]) rank += a.key[j] < k;
-        const u64 p = (u64)row_start[row] + rank;
+        const u64 p = (u64)r0 + rank;
         if (p >= a.cap) continue;   // only after an overflow, when the run is repeated
+        const int4 r = a.rec[i];
+        xyz[3 * p + 0] = r.x;
+        xyz[3 * p + 1] = r.y;
+        xyz[3 * p + 2] = r.z;
+        pulse[p] = r.w;
+    }
+}
+
+// Placement where rows are crowded.  First every grain takes a slot of its row's
+// part of one array (x << 32 | grain; the row counts count down to 0) ...
+__global__ void k_fr_bucket(FrArgs a, const u32 *row_start, u64 *bucket) {
+    griddep_launch();
+    griddep_wait();
+    const u64 n = min(a.ctl->n_grains, a.cap), stride = (u64)gridDim.x * blockDim.x;
+    for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const u64 k = a.key[i], row = k >> 12;
+        const u64 p = (u64)row_start[row] + atomicSub(&a.row_count[row], 1u) - 1u;
+        bucket[p] = ((k & 4095u) << 32) | i;
+    }
+}
+
+// ... then it counts the smaller x of its row in that part.  Neighbouring lanes
+// are mostly of one row and read the same entries.
+__global__ void k_fr_rank(FrArgs a, const u32 *row_start, const u64 *bucket, int *xyz, int *pulse) {
+    griddep_launch();
+    griddep_wait();
+    const u64 n = min(a.ctl->n_grains, a.cap), stride = (u64)gridDim.x * blockDim.x;
+    for (u64 q = (u64)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += stride) {
+        const u64 e = bucket[q], i = e & 0xffffffffu, row = a.key[i] >> 12;
+        const u32 r0 = row_start[row], r1 = row_start[row + 1];
+        u64 p = r0;
+        for (u32 j = r0; j < r1; ++j) p += bucket[j] < e;   // no two grains of a row share x
         const int4 r = a.rec[i];
         xyz[3 * p + 0] = r.x;
         xyz[3 * p + 1] = r.y;
@@ -328,6 +375,7 @@ struct FramesRT {
     Ctx *ctx;
     et_frame_params p;
     Group g_tab, g_raw, g_out, g_ctl;
+    Group g_bucket;   // for stacks with crowded rows, once there was one
     unsigned char *gain = nullptr, *thr = nullptr, *cut = nullptr;
     unsigned short *cal = nullptr;
     FrCtl *ctl = nullptr;
@@ -364,6 +412,7 @@ struct FramesRT {
         g_raw.release(ctx);
         g_out.release(ctx);
         g_ctl.release(ctx);
+        g_bucket.release(ctx);
     }
 
     size_t pixels() const { return (size_t)p.width * p.height; }
@@ -433,10 +482,7 @@ struct FramesRT {
         return ET_OK;
     }
 
-    et_status enqueue(cudaStream_t st) {
-        cudaMemsetAsync(ctl, 0, sizeof(FrCtl), st);
-        cudaMemsetAsync(row_count, 0, sizeof(u32) * rows(), st);
-        cudaMemsetAsync(row_head, 0xFF, sizeof(u32) * rows(), st);
+    FrArgs args() const {
         FrArgs a;
         memset(&a, 0, sizeof a);
         a.W = p.width;
@@ -452,7 +498,6 @@ struct FramesRT {
         a.chunks = (p.width + 15) / 16;
         while (a.lc < 4 && (1 << a.lc) < a.chunks) ++a.lc;
         a.tiles_x = (a.chunks + (1 << a.lc) - 1) >> a.lc;
-        const int tile_h = FT >> a.lc, tiles_y = (p.height + tile_h - 1) / tile_h;
         a.raw = d_raw;
         a.gain = gain;
         a.thr = thr;
@@ -466,6 +511,15 @@ struct FramesRT {
         a.cap = cap;
         a.row_count = row_count;
         a.row_head = row_head;
+        return a;
+    }
+
+    et_status enqueue(cudaStream_t st) {
+        cudaMemsetAsync(ctl, 0, sizeof(FrCtl), st);
+        cudaMemsetAsync(row_count, 0, sizeof(u32) * rows(), st);
+        cudaMemsetAsync(row_head, 0xFF, sizeof(u32) * rows(), st);
+        FrArgs a = args();
+        const int tile_h = FT >> a.lc, tiles_y = (p.height + tile_h - 1) / tile_h;
         cudaEventRecord(ev[1], st);
         // the depth in as few pieces as give the device 8 blocks per SM
         const long long tiles = (long long)a.tiles_x * tiles_y * V;
@@ -477,10 +531,28 @@ struct FramesRT {
         cudaEventRecord(ev[2], st);
         exclusive_scan_u32(row_count, row_start, (long long)rows(), temp, st, &ctl->error, FRB_TIMEOUT, ctl->bar);
         launch_dep(k_fr_place, dim3(152 * 4), dim3(256), 0, st, a, row_start, xyz, pulse, view_off);
-        if (stage) launch_dep(k_fr_publish, dim3(16), dim3(512), 0, st, a, (const int *)xyz, (const int *)pulse, (const u32 *)view_off, stage);
+        publish(a, st);
         launches = stage ? 4 : 3;   // recognition, the scan of the row counts, placement, publication
         cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? ET_OK : cuda_fail(e, "front-end launch");
+    }
+
+    void publish(const FrArgs &a, cudaStream_t st) {
+        if (stage) launch_dep(k_fr_publish, dim3(16), dim3(512), 0, st, a, (const int *)xyz, (const int *)pulse, (const u32 *)view_off, stage);
+    }
+
+    // The placement again, for rows too long to walk.
+    et_status place_crowded(cudaStream_t st) {
+        if (!g_bucket.reserve(ctx, sizeof(u64) * std::max<u64>(n_grains(), 1)))
+            return fail(ET_ERR_OOM, "row order of %llu grains", (unsigned long long)n_grains());
+        const FrArgs a = args();
+        u64 *bucket = (u64 *)g_bucket.base;
+        launch_dep(k_fr_bucket, dim3(ctx->sms * 4), dim3(256), 0, st, a, (const u32 *)row_start, bucket);
+        launch_dep(k_fr_rank, dim3(ctx->sms * 8), dim3(256), 0, st, a, (const u32 *)row_start, (const u64 *)bucket, xyz, pulse);
+        publish(a, st);
+        launches += stage ? 3 : 2;
+        cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? ET_OK : cuda_fail(e, "row order launch");
     }
 
     et_status run(const unsigned char *raw, int nv, bool on_device, cudaStream_t st) {
@@ -525,6 +597,7 @@ struct FramesRT {
     et_status settle() {
         if (!ran) return fail(ET_ERR_NOT_READY, "nothing has been run");
         if (settled) return run_status;
+        bool placed = false;   // this run's crowded rows
         for (int attempt = 0; attempt < 4; ++attempt) {
             cudaError_t e = cudaEventSynchronize(ev[3]);
             if (e != cudaSuccess) return run_status = cuda_fail(e, "front-end run");
@@ -534,6 +607,17 @@ struct FramesRT {
             if (hctl.error & FRB_TIMEOUT) {
                 settled = true;
                 return run_status = fail(ET_ERR_TIMEOUT, "a frame load did not complete in time");
+            }
+            if ((hctl.error & (FRB_OVF | FRB_CROWDED)) == FRB_CROWDED && !placed) {
+                et_status s = place_crowded(ctx->stream);
+                cudaEventRecord(ev[3], ctx->stream);
+                if (s != ET_OK) {
+                    settled = g_bucket.base != nullptr;   // without it nothing was launched: the next call tries again
+                    return run_status = s;
+                }
+                placed = true;
+                --attempt;
+                continue;
             }
             if (!(hctl.error & FRB_OVF)) {
                 cudaEventElapsedTime(&kernel_ms, ev[1], ev[2]);
