@@ -573,11 +573,13 @@ __device__ void jacobi3f(float A[3][3], float V[3][3]) {
 
 // One warp per accepted track: exact integer moments about the lo seed grain,
 // FP32 principal axis, member projections, and the members (caller indices) in
-// ascending order: a track of up to FIT_SORT of them is sorted by rank (each
-// member counts the smaller ones) in the warp's shared memory, longer ones are
-// left to k_long_members.  A global sort of all members by (track, index)
-// instead took 39 us on a 28k-grain view with 344 tracks.
-constexpr int FIT_T = 256, FIT_SORT = 512;
+// ascending order: a track of up to FIT_RANK of them is sorted by rank (each
+// member counts the smaller ones) in the warp's shared memory, one of up to
+// FIT_SORT by a bitonic network there (one track of 512: the stage 89 us by rank,
+// 40 by the network), longer ones are left to k_long_members.  A global sort of
+// all members by (track, index) instead took 39 us on a 28k-grain view with 344
+// tracks.
+constexpr int FIT_T = 256, FIT_RANK = 64, FIT_SORT = 512;
 
 __global__ void __launch_bounds__(FIT_T) k_fit(Batch b, Work w, Out o) {
     __shared__ int ids[FIT_T / 32][FIT_SORT];
@@ -615,13 +617,31 @@ __global__ void __launch_bounds__(FIT_T) k_fit(Batch b, Work w, Out o) {
             written += __popc(bal);
         }
         __syncwarp();
-        if (written <= FIT_SORT) {
+        if (written <= FIT_RANK) {
             for (u32 k = lane; k < written; k += 32) {
                 const int mine = id[k];
                 u32 rank = 0;
                 for (u32 j = 0; j < written; ++j) rank += id[j] < mine;
                 o.out_members[obase + rank] = mine;
             }
+        } else if (written <= FIT_SORT) {
+            u32 n2 = 2 * FIT_RANK;
+            while (n2 < written) n2 *= 2;
+            for (u32 k = written + lane; k < n2; k += 32) id[k] = 0x7fffffff;
+            __syncwarp();
+            for (u32 size = 2; size <= n2; size *= 2)
+                for (u32 step = size / 2; step > 0; step /= 2) {
+#pragma unroll 4
+                    for (u32 i = lane; i < n2 / 2; i += 32) {
+                        const u32 x = 2 * i - (i & (step - 1)), y = x + step;
+                        const int a = id[x], c2 = id[y];
+                        const bool swap = (a > c2) == ((x & size) == 0);
+                        id[x] = swap ? c2 : a;
+                        id[y] = swap ? a : c2;
+                    }
+                    __syncwarp();
+                }
+            for (u32 k = lane; k < written; k += 32) o.out_members[obase + k] = id[k];
         } else if (lane == 0) {
             o.long_tracks[atomicAdd(&b.ctl->n_long, 1u)] = (int)t;
         }
@@ -700,34 +720,40 @@ __global__ void __launch_bounds__(FIT_T) k_fit(Batch b, Work w, Out o) {
 }
 
 // Members of the tracks longer than FIT_SORT, one block per track: a bitmap of
-// the caller indices (below 2^21), half of the range at a time, whose set bits
-// are written out in order.
+// the caller indices (below 2^rbits), LONG_BITS of them at a time, whose set bits
+// are written out in order.  A thread scans consecutive words, so word w lies at w
+// + w / 32: at w the lanes of a warp met in one bank.  200 tracks of 600 took the
+// stage 0.88 ms over all 2^21 indices by 16 blocks, and take 0.09 ms.
 constexpr int LONG_T = 1024, LONG_BITS = 1 << 20;
+
+__host__ __device__ constexpr u32 long_word(u32 w) { return w + (w >> 5); }
+__host__ __device__ inline u32 long_words(int rbits) { return max(1u, min((u32)LONG_BITS, 1u << rbits) / 32u); }
 
 __global__ void __launch_bounds__(LONG_T) k_long_members(Batch b, Work w, Out o) {
     griddep_launch();
     griddep_wait();
     if (input_failed(b.ctl)) return;
-    extern __shared__ __align__(16) u32 bits[];   // LONG_BITS / 32
+    extern __shared__ __align__(16) u32 bits[];   // long_word(long_words(rbits)) of them
     __shared__ u32 wsum[LONG_T / 32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    constexpr int PER = LONG_BITS / 32 / LONG_T;   // words a thread scans
+    const u32 nw = long_words(b.rbits), per = (nw + LONG_T - 1) / LONG_T;   // words, and those a thread scans
+    const u32 w0 = min(nw, threadIdx.x * per), w1 = min(nw, w0 + per);
     for (u32 l = blockIdx.x; l < b.ctl->n_long; l += gridDim.x) {
         const int t = o.long_tracks[l], c = o.acc[t];
         const u64 m0 = w.c_moff[c], m1 = m0 + w.c_cnt[c];
         u64 obase = o.trk_moff[t];
-        for (int base = 0; base < (1 << 21); base += LONG_BITS) {
-            for (int i = threadIdx.x; i < LONG_BITS / 32; i += LONG_T) bits[i] = 0;
+        for (int base = 0; base < 1 << b.rbits; base += LONG_BITS) {
+            for (u32 i = threadIdx.x; i < nw; i += LONG_T) bits[long_word(i)] = 0;
             __syncthreads();
             for (u64 m = m0 + threadIdx.x; m < m1; m += LONG_T) {
                 const int g = w.members[m];
                 if (w.owner[g] != c) continue;
                 const int i = b.gr[g].w - base;
-                if (i >= 0 && i < LONG_BITS) atomicOr(&bits[i >> 5], 1u << (i & 31));
+                if (i >= 0 && i < LONG_BITS) atomicOr(&bits[long_word((u32)i >> 5)], 1u << (i & 31));
             }
             __syncthreads();
             u32 n = 0;
-            for (int k = 0; k < PER; ++k) n += __popc(bits[threadIdx.x * PER + k]);
+            for (u32 k = w0; k < w1; ++k) n += __popc(bits[long_word(k)]);
             u32 incl = n;
 #pragma unroll
             for (int s = 1; s < 32; s <<= 1) {
@@ -742,10 +768,8 @@ __global__ void __launch_bounds__(LONG_T) k_long_members(Batch b, Work w, Out o)
                 total += wsum[k];
             }
             u64 pos = obase + before + incl - n;
-            for (int k = 0; k < PER; ++k) {
-                const int word = threadIdx.x * PER + k;
-                for (u32 x = bits[word]; x; x &= x - 1) o.out_members[pos++] = base + word * 32 + __ffs(x) - 1;
-            }
+            for (u32 k = w0; k < w1; ++k)
+                for (u32 x = bits[long_word(k)]; x; x &= x - 1) o.out_members[pos++] = base + (int)k * 32 + __ffs(x) - 1;
             obase += total;
             __syncthreads();
         }
@@ -791,7 +815,8 @@ int bits_for(unsigned long long maxval) {
 }  // namespace
 
 int merge_grid_blocks(int device) {
-    cudaFuncSetAttribute(k_long_members, cudaFuncAttributeMaxDynamicSharedMemorySize, LONG_BITS / 8);
+    cudaFuncSetAttribute(k_long_members, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(long_word(LONG_BITS / 32) * sizeof(u32)));
     cudaFuncSetAttribute(k_acc_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(ACC_SMALL * (sizeof(u64) + sizeof(u32))));
     int sms = 0, per_sm = 0;
@@ -828,7 +853,9 @@ void launch_single_pass(const Batch &b, const Work &w, cudaStream_t st) {
 
 static void launch_fit(const Batch &b, const Work &w, const Out &o, cudaStream_t st) {
     launch_dep(k_fit, dim3(sm_count() * 4), dim3(FIT_T), 0, st, b, w, o);
-    launch_dep(k_long_members, dim3(std::min(16u, sm_count())), dim3(LONG_T), (size_t)(LONG_BITS / 8), st, b, w, o);
+    // a block for every track that can be this long, one at least
+    const unsigned g = (unsigned)std::min<long long>(sm_count(), std::max(1, b.N / (FIT_SORT + 1)));
+    launch_dep(k_long_members, dim3(g), dim3(LONG_T), long_word(long_words(b.rbits)) * sizeof(u32), st, b, w, o);
 }
 
 // Accepted list sorted by (view, key); per-view track offsets; member offsets;
