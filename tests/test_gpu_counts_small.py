@@ -1,0 +1,33 @@
+"""The allocation-free counts of tiny views with lists of pairs around the numbers where a warp's first share
+is the whole work (32 pairs for each of four blocks of eight warps an SM) and where shares are taken on."""
+import numpy as np
+import pytest
+
+from paper_1311_5334_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("grains", [2, 120])
+def test_pair_lists_around_one_share_a_warp(oracle_mod, grains):
+    import torch
+    from paper_1311_5334_gb300 import et
+
+    v = synth.make_view(19, n_fog=max(2, grains - 40), n_through=0 if grains == 2 else 1)
+    xyz = v.xyz[:grains]
+    p = synth.params(v.extent)
+    with oracle_mod.Oracle(xyz, v.extent, p["seed_min"], p["seed_max"], p["tube_r"], p["min_hits"]) as o:
+        i, j = np.meshgrid(np.arange(len(xyz)), np.arange(len(xyz)), indexing="ij")
+        near = (i != j) & (np.abs(xyz[i] - xyz[j]) < p["seed_max"]).all(-1)
+        table = np.full(i.shape, -1, dtype=np.int64)
+        if near.any():
+            table[near] = o.count_pairs(i[near], j[near])
+    with et.Context(0) as ctx:
+        warps = ctx.info()["sm_count"] * 4 * 8
+    d_xyz = torch.from_numpy(np.ascontiguousarray(xyz)).cuda()
+    rng = np.random.default_rng(grains)
+    for count in [n + k for n in (4 * warps, 32 * warps, 64 * warps) for k in (-1, 0, 1)]:
+        pairs = rng.integers(0, len(xyz), (count, 2)).astype(np.int32)
+        out = torch.full((count,), -7, dtype=torch.int32, device="cuda")
+        et.tube_count_noalloc(d_xyz, p, torch.from_numpy(pairs).cuda(), out)
+        assert np.array_equal(out.cpu().numpy(), table[pairs[:, 0], pairs[:, 1]])
