@@ -39,9 +39,12 @@ struct Ctx {
     // page-locked stages given back by batches and front ends, at most STAGE_POOL
     static constexpr size_t STAGE_POOL = 16;
     std::mutex stage_mu;
-    std::vector<void *> stages[2];
+    std::vector<void *> stages[2];   // never beyond their first capacity: give_stage runs in destructors
     void *take_stage(int kind, size_t bytes);
     void give_stage(int kind, void *p);
+    Ctx() {
+        for (auto &s : stages) s.reserve(STAGE_POOL);
+    }
     ~Ctx();
     void *dalloc(size_t bytes);
     void dfree(void *p);
