@@ -485,6 +485,7 @@ size_t BatchRT::footprint_with(const size_t sizes[NGROUP]) const {
 }
 
 void BatchRT::release_groups() {
+    laid = false;
     for (int k = 0; k < NGROUP; ++k) group(k)->release(ctx);
 }
 
