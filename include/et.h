@@ -169,8 +169,8 @@ typedef struct {
     int32_t profiled;       /* 1 if stage_ms holds timings of the last run */
     /* with profiling on: CUDA-event time of each stage of the last run, ms:
      * 0 canonical order + cell list, 1 (empty: the seeds are generated inside
-     * the tube-count kernel), 2 seeds + tube counts, 3 candidate keys + member
-     * lists, 4 merge, 5 output (order, fit, members) */
+     * the tube-count kernel), 2 seeds + tube counts + candidates, 3 member lists,
+     * 4 merge, 5 output (order, fit, members) */
     float stage_ms[6];
     int64_t n_pair_tests;   /* seed-window tests the seed generator made (grain pairs examined) */
 } et_stats;

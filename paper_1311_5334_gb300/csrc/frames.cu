@@ -54,14 +54,13 @@ struct FrCtl {
 
 struct FrArgs {
     int W, H, D, P, V;
-    int T;
     int num[3], den[3];
     int chunks;                 // 16-pixel chunks per row
     int zb;                     // frames of a block, a multiple of ZC
     int lc, tiles_x;            // a tile is 2^lc chunks wide and FT / 2^lc rows high; tiles per row
     const unsigned char *raw;
-    const unsigned char *gain, *thr, *cut;   // padded tables: pixel (x, y) at (y + 1) * TP + x + 16
-    const unsigned short *cal;               // gain | thr << 8, same layout
+    const unsigned char *cut;       // padded tables: pixel (x, y) at (y + 1) * TP + x + 16
+    const unsigned short *cal;      // gain | thr << 8, same layout
     int TP;
     FrCtl *ctl;
     u64 *key;                   // row << 12 | x
@@ -73,7 +72,10 @@ struct FrArgs {
 };
 
 // Page-locked host memory that the last kernel of a run writes (as Stage of the
-// tracking): control block, view offsets and grains where they are few.
+// tracking): control block, view offsets and grains where they are few.  A full
+// stack of 1,600, 6,400 and 11,900 grains takes 83, 87 and 90 us with copies and 72,
+// 78 and 85 us with publication; from some 18,000 grains on the copies are faster
+// (34,000 grains: 93 and, in a copy of this code with a larger limit, 109 us).
 constexpr u32 FSTAGE_GRAINS = 16384, FSTAGE_VIEWS = 1024;
 struct FrStage {
     FrCtl ctl;
@@ -452,7 +454,7 @@ struct FramesRT {
         if (e != cudaSuccess) return cuda_fail(e, "calibration upload");
         // zero gain outside the frame gives a zero cutoff there
         const int n = (int)table_bytes();
-        k_cutoff<<<std::min((n + 255) / 256, 152 * 8), 256, 0, st>>>(gain, thr, cut, cal, n, p.grain_threshold);
+        k_cutoff<<<std::min((n + 255) / 256, ctx->sms * 8), 256, 0, st>>>(gain, thr, cut, cal, n, p.grain_threshold);
         e = cudaStreamSynchronize(st);   // the caller may free its tables on return
         return e == cudaSuccess ? ET_OK : cuda_fail(e, "cutoff table");
     }
@@ -490,7 +492,6 @@ struct FramesRT {
         a.D = p.depth;
         a.P = p.row_pitch;
         a.V = V;
-        a.T = p.grain_threshold;
         for (int k = 0; k < 3; ++k) {
             a.num[k] = p.pitch_num[k];
             a.den[k] = p.pitch_den[k];
@@ -499,8 +500,6 @@ struct FramesRT {
         while (a.lc < 4 && (1 << a.lc) < a.chunks) ++a.lc;
         a.tiles_x = (a.chunks + (1 << a.lc) - 1) >> a.lc;
         a.raw = d_raw;
-        a.gain = gain;
-        a.thr = thr;
         a.cut = cut;
         a.cal = cal;
         a.TP = table_pitch();
@@ -524,13 +523,13 @@ struct FramesRT {
         // the depth in as few pieces as give the device 8 blocks per SM
         const long long tiles = (long long)a.tiles_x * tiles_y * V;
         const int steps = (p.depth + ZC - 1) / ZC;
-        const int pieces = (int)std::min<long long>(steps, std::max<long long>(1, (152 * 8 + tiles - 1) / tiles));
+        const int pieces = (int)std::min<long long>(steps, std::max<long long>(1, ((long long)ctx->sms * 8 + tiles - 1) / tiles));
         a.zb = (steps + pieces - 1) / pieces * ZC;
         launch_dep(k_recognize, dim3((unsigned)(a.tiles_x * tiles_y), (unsigned)((p.depth + a.zb - 1) / a.zb), (unsigned)V),
                    dim3(FT), 0, st, a);
         cudaEventRecord(ev[2], st);
         exclusive_scan_u32(row_count, row_start, (long long)rows(), temp, st, &ctl->error, FRB_TIMEOUT, ctl->bar);
-        launch_dep(k_fr_place, dim3(152 * 4), dim3(256), 0, st, a, row_start, xyz, pulse, view_off);
+        launch_dep(k_fr_place, dim3(ctx->sms * 4), dim3(256), 0, st, a, row_start, xyz, pulse, view_off);
         publish(a, st);
         launches = stage ? 4 : 3;   // recognition, the scan of the row counts, placement, publication
         cudaError_t e = cudaGetLastError();
@@ -606,7 +605,7 @@ struct FramesRT {
             if (e != cudaSuccess) return run_status = cuda_fail(e, "control block read");
             if (hctl.error & FRB_TIMEOUT) {
                 settled = true;
-                return run_status = fail(ET_ERR_TIMEOUT, "a frame load did not complete in time");
+                return run_status = fail(ET_ERR_TIMEOUT, "the scan of the row counts did not complete in time");
             }
             if ((hctl.error & (FRB_OVF | FRB_CROWDED)) == FRB_CROWDED && !placed) {
                 et_status s = place_crowded(ctx->stream);
