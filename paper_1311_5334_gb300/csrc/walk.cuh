@@ -73,7 +73,11 @@ __device__ __forceinline__ float3 slab_coeffs(float a, float w, float iw, float 
 }
 
 // Resolves the cover geometry of the line through ga and gb into q and
-// returns its number of items (outer slabs).
+// returns its number of items (outer slabs).  There is at least one: a lies in the
+// view, so t0 < 0 < t1 (pad > 0 keeps the signs), so [a - pad, a + pad] lies within
+// the range of every axis, and its cells from (a - pad) / cell to (a + pad) / cell hold
+// a's, as the rounding of either (below 2^21 x 2^-22) is less than pad.  warp_items
+// counts on that.
 __device__ __forceinline__ int seed_setup(const Batch &b, int4 ga, int4 gb, int view, SeedSm &q) {
     const float pad = (float)b.r + COVER_PAD;
     const int wxi = gb.x - ga.x, wyi = gb.y - ga.y, wzi = gb.z - ga.z;
