@@ -334,10 +334,15 @@ extern "C" et_status et_tube_count_noalloc(const int32_t *d_xyz, int64_t n, cons
     long long nx = 0, ny = 0;
     for (int tries = 0; tries < 64; ++tries) {
         nx = ny = 1;
-        for (int k = 0; k < 3; ++k) b.cs[k] = (int)std::min<double>(std::max(1.0, std::round(s0 * AUTO_CELL[k])), b.ext[k]);
-        b.csy[0] = std::min(b.cs[1], b.ext[0]);
-        b.csy[1] = std::min(b.cs[0], b.ext[1]);
-        b.csy[2] = b.cs[2];
+        // the second list's edges along x and y are the first one's along y and x as
+        // chosen, not as cut to a thin extent: either list comes down to one cell
+        auto edge = [&](int shape, int axis) {
+            return (int)std::min<double>(std::max(1.0, std::round(s0 * AUTO_CELL[shape])), b.ext[axis]);
+        };
+        for (int k = 0; k < 3; ++k) {
+            b.cs[k] = edge(k, k);
+            b.csy[k] = edge(k == 2 ? 2 : 1 - k, k);
+        }
         for (int k = 0; k < 3; ++k) {
             b.nc[k] = (b.ext[k] + b.cs[k] - 1) / b.cs[k];
             b.ncy[k] = (b.ext[k] + b.csy[k] - 1) / b.csy[k];

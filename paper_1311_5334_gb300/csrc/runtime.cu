@@ -230,7 +230,7 @@ void BatchRT::choose_cells() {
     if (lay(s, AUTO_CELL) <= room) return;
     static const double mean_shape[3] = {0.22, 1.1, 1.1};
     const double limit = std::max(room, lay(edge(V > 0 ? (double)N / V : 1.0), mean_shape));
-    while (lay(s, AUTO_CELL) > limit) s *= 1.1;   // ends: one cell a view is within the limit
+    while (lay(s, AUTO_CELL) > limit) s *= 1.1;   // ends: no edge is then below the mean shape's
 }
 
 // One origin per work ticket while a batch is small enough that the last

@@ -31,3 +31,25 @@ def test_pair_lists_around_one_share_a_warp(oracle_mod, grains):
         out = torch.full((count,), -7, dtype=torch.int32, device="cuda")
         et.tube_count_noalloc(d_xyz, p, torch.from_numpy(pairs).cuda(), out)
         assert np.array_equal(out.cpu().numpy(), table[pairs[:, 0], pairs[:, 1]])
+
+
+@pytest.mark.parametrize("extent", [(1 << 20, 2, 3), (3, 1 << 20, 2), (2, 3, 1 << 20), (1 << 20, 1, 1), (700000, 40, 300000)])
+def test_long_thin_views(oracle_mod, extent):
+    """Extents of which the cell list with rows along x, or the one along y, has most of its cells."""
+    import torch
+    from paper_1311_5334_gb300 import et
+
+    rng = np.random.default_rng(sum(extent))
+    xyz = np.unique(rng.integers(0, extent, (3000, 3)), axis=0).astype(np.int32)
+    xyz = np.ascontiguousarray(xyz[rng.permutation(len(xyz))])
+    p = synth.params(extent, seed_min=0, seed_max=1000, tube_r=3)
+    order = np.lexsort(xyz.T)
+    i = rng.integers(0, len(xyz) - 4, 5000)
+    pairs = np.stack([order[i], order[i + rng.integers(1, 4, 5000)]], 1).astype(np.int32)
+    good = (np.abs(xyz[pairs[:, 0]] - xyz[pairs[:, 1]]) < p["seed_max"]).all(1)
+    want = np.full(len(pairs), -1, dtype=np.int64)
+    with oracle_mod.Oracle(xyz, extent, p["seed_min"], p["seed_max"], p["tube_r"], p["min_hits"]) as o:
+        want[good] = o.count_pairs(pairs[good, 0].astype(np.int64), pairs[good, 1].astype(np.int64))
+    out = torch.full((len(pairs),), -7, dtype=torch.int32, device="cuda")
+    et.tube_count_noalloc(torch.from_numpy(xyz).cuda(), p, torch.from_numpy(pairs).cuda(), out)
+    assert np.array_equal(out.cpu().numpy(), want)
