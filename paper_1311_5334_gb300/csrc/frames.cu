@@ -211,10 +211,10 @@ __global__ void __launch_bounds__(FT, 4) k_recognize(const __grid_constant__ FrA
     griddep_launch();
     griddep_wait();
     __shared__ u32 queue[QCAP];   // thread | pixel << 8 | frame << 12
-    __shared__ u32 queued;
+    __shared__ u32 queued, passed;
     static_assert(FT == 256, "bits of a queue entry");
     const int tid = threadIdx.x;
-    if (tid == 0) queued = 0;
+    if (tid == 0) queued = passed = 0;
     __syncthreads();
     const int tx0 = (blockIdx.x % a.tiles_x) << a.lc, ty0 = (blockIdx.x / a.tiles_x) * (FT >> a.lc);
     const int chunk = tx0 + (tid & ((1 << a.lc) - 1)), y = ty0 + (tid >> a.lc);
@@ -223,20 +223,32 @@ __global__ void __launch_bounds__(FT, 4) k_recognize(const __grid_constant__ FrA
     const bool mine = chunk < a.chunks && y < a.H;
     const unsigned char *src = a.raw + ((size_t)v * a.D + z0) * frame + (size_t)y * a.P + chunk * 16;
     u32 cv[4] = {0u, 0u, 0u, 0u};
-    // queues the pixels of frame kz below their cutoffs
-    auto scan = [&](uint4 r, int kz) {
-        // per byte raw < cutoff, four bytes a word (SWAR): with the byte's high
-        // bits ra, ca and d = (raw | 0x80) - (cutoff & 0x7f) (no borrow between
-        // bytes), raw < cutoff iff (!ra & ca) | (ra == ca & !d7)
-        const u32 rw[4] = {r.x, r.y, r.z, r.w};
+    u32 ncand = 0;
+    // per byte a < b, four bytes a word (SWAR): with the bytes' high bits a7, b7 and
+    // d = (a | 0x80) - (b & 0x7f) (no borrow between bytes), a < b iff
+    // (!a7 & b7) | (a7 == b7 & !d7)
+    auto below = [](u32 a, u32 b) {
+        const u32 d = (a | 0x80808080u) - (b & 0x7f7f7f7fu);
+        return ((~a & b) | (~(a ^ b) & ~d)) & 0x80808080u;
+    };
+    auto bits = [](const u32 (&w)[4]) {   // bit 8 j + k: byte j of word k
+        return (w[0] >> 7) | (w[1] >> 6) | (w[2] >> 5) | (w[3] >> 4);
+    };
+    // queues the pixels r of frame kz below their cutoffs, except those that are no
+    // brighter in the frame before (p): calibrated alike and filtered without increasing
+    // in the raw value, their pulse there is no smaller, which rules a maximum out.
+    // Without that a dark stack queued every voxel.
+    auto scan = [&](uint4 r, uint4 p, int kz) {
+        const u32 rw[4] = {r.x, r.y, r.z, r.w}, pw[4] = {p.x, p.y, p.z, p.w};
         u32 lt[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const u32 d = (rw[k] | 0x80808080u) - (cv[k] & 0x7f7f7f7fu);
-            lt[k] = ((~rw[k] & cv[k]) | (~(rw[k] ^ cv[k]) & ~d)) & 0x80808080u;
-        }
+        for (int k = 0; k < 4; ++k) lt[k] = below(rw[k], cv[k]);
         if (lt[0] | lt[1] | lt[2] | lt[3]) {
-            u32 m = (lt[0] >> 7) | (lt[1] >> 6) | (lt[2] >> 5) | (lt[3] >> 4);   // bit 8 j + k: byte j of word k
+            ncand += (u32)__popc(bits(lt));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) lt[k] &= below(rw[k], pw[k]);
+            u32 m = bits(lt);
+            if (m == 0) return;
             u32 s = atomicAdd(&queued, (u32)__popc(m));
             for (; m && s < QCAP; m &= m - 1, ++s) {
                 const int bit = __ffs(m) - 1, px = 4 * (bit & 7) + (bit >> 3);
@@ -258,6 +270,7 @@ __global__ void __launch_bounds__(FT, 4) k_recognize(const __grid_constant__ FrA
         cv[1] = c4.y;
         cv[2] = c4.z;
         cv[3] = c4.w;
+        uint4 before = make_uint4(~0u, ~0u, ~0u, ~0u);   // the piece's first frame: nothing is ruled out
         for (int z = 0; z < nz; z += ZC) {
             uint4 r[ZC];
 #pragma unroll
@@ -265,22 +278,30 @@ __global__ void __launch_bounds__(FT, 4) k_recognize(const __grid_constant__ FrA
                 if (z + k < nz) r[k] = __ldg((const uint4 *)(src + (size_t)(z + k) * frame));
 #pragma unroll
             for (int k = 0; k < ZC; ++k)
-                if (z + k < nz) scan(r[k], z + k);
+                if (z + k < nz) scan(r[k], k ? r[k - 1] : before, z + k);
+            before = r[ZC - 1];
         }
     }
+    ncand = __reduce_add_sync(0xffffffffu, ncand);
+    if ((tid & 31) == 0 && ncand) atomicAdd(&passed, ncand);
     __syncthreads();
     const u32 all = queued;
-    if (tid == 0 && all) atomicAdd(&a.ctl->n_cand, (u64)all);
+    if (tid == 0 && passed) atomicAdd(&a.ctl->n_cand, (u64)passed);
     if (all <= QCAP) {
         test_queue(all);
         return;
     }
     // a crowded tile: again, a frame at a time (its candidates always fit)
+    uint4 before = make_uint4(~0u, ~0u, ~0u, ~0u);
     for (int k = 0; k < nz; ++k) {
         __syncthreads();
         if (tid == 0) queued = 0;
         __syncthreads();
-        if (mine) scan(__ldg((const uint4 *)(src + (size_t)k * frame)), k);
+        if (mine) {
+            const uint4 r = __ldg((const uint4 *)(src + (size_t)k * frame));
+            scan(r, before, k);
+            before = r;
+        }
         __syncthreads();
         test_queue(queued);
     }
