@@ -207,10 +207,11 @@ __global__ void __launch_bounds__(NA_W * 32, 4) k_na_tube(Batch b, const int *xy
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const bool bad_view = *(volatile u32 *)&s.ctl->bad != 0;
     const long long nwarps = (long long)gridDim.x * NA_W;
-    const int lines = (int)max(4ll, min(32ll, (n_pairs + nwarps - 1) / nwarps));
-    // a warp's first pairs follow from its number, the next ones (if all warps' first
-    // are not the whole list) are taken from the counter: 100k pairs of 115 grains
-    // 29 us, 34 with every pair taken from it
+    const int lines = (int)max(4ll, min(32ll, (n_pairs + 2 * nwarps - 1) / (2 * nwarps)));
+    // a warp's first pairs follow from its number, the next ones, about half of a list
+    // that would do with one share a warp, from the counter, as pairs differ in
+    // their grains: 100k pairs of 115 grains 30 us, 34 with every pair taken from
+    // the counter; 75k pairs of 10k crowded grains 232 us, 322 with one share a warp
     u64 k0 = ((u64)blockIdx.x * NA_W + wib) * (u64)lines;
     const u64 first = (u64)nwarps * (u64)lines;
     while (k0 < (u64)n_pairs) {
@@ -231,17 +232,19 @@ __global__ void __launch_bounds__(NA_W * 32, 4) k_na_tube(Batch b, const int *xy
         // past the others
         const unsigned gm = __ballot_sync(0xffffffffu, good);
         const int slot = __popc(gm & ((1u << lane) - 1u));
-        scount[wib][lane] = 0;
-        if (good) {
-            SeedSm q;
-            nit[wib][slot] = seed_setup(b, a, c, 0, q);
-            sp[wib].put(slot, q);
+        if (gm) {
+            scount[wib][lane] = 0;
+            if (good) {
+                SeedSm q;
+                nit[wib][slot] = seed_setup(b, a, c, 0, q);
+                sp[wib].put(slot, q);
+            }
+            __syncwarp();
+            u32 tests = 0;
+            warp_items<true, true, WALK_SERIAL>(b, sp[wib], tbl[wib], lane < __popc(gm) ? nit[wib][lane] : 0, tests,
+                                                scount[wib], [&](int own, int4) { atomicAdd(&scount[wib][own], 1u); });
+            __syncwarp();
         }
-        __syncwarp();
-        u32 tests = 0;
-        warp_items<true, true, WALK_SERIAL>(b, sp[wib], tbl[wib], lane < __popc(gm) ? nit[wib][lane] : 0, tests,
-                                            scount[wib], [&](int own, int4) { atomicAdd(&scount[wib][own], 1u); });
-        __syncwarp();
         if (mine) counts[k] = good ? (int)scount[wib][slot] : -1;
         __syncwarp();
         if (first >= (u64)n_pairs) break;
@@ -331,6 +334,11 @@ extern "C" et_status et_tube_count_noalloc(const int32_t *d_xyz, int64_t n, cons
     b.smax = params->seed_max;
     const double vol = (double)b.ext[0] * b.ext[1] * b.ext[2];
     double s0 = std::cbrt(1.4 * vol / (double)std::max<int64_t>(n, 1));
+    // no more cells than the pairs repay: one block scans a list's cells, some 0.3 us a
+    // thousand.  At half a cell a pair and at all that fit, us a call: 65,536 grains with
+    // 1, 1,000, 30,000 and 100,000 pairs 37 and 113, 85 and 124, 81 and 130, 122 and 154;
+    // 21,783 grains of a thin extent with one pair 35 and 166
+    const long long most_cells = std::min<long long>(NA_LIST_CELLS, std::max<long long>(4096, n_pairs / 2));
     long long nx = 0, ny = 0;
     for (int tries = 0; tries < 64; ++tries) {
         nx = ny = 1;
@@ -351,7 +359,7 @@ extern "C" et_status et_tube_count_noalloc(const int32_t *d_xyz, int64_t n, cons
             nx *= b.nc[k];
             ny *= b.ncy[k];
         }
-        if (std::max(nx, ny) <= NA_LIST_CELLS) break;
+        if (std::max(nx, ny) <= most_cells) break;
         s0 *= 1.26;
     }
     if (std::max(nx, ny) > NA_LIST_CELLS) return fail(ET_ERR_INVALID_ARG, "no cell grid fits the fixed scratch limit");
