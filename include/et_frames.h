@@ -61,8 +61,8 @@ typedef struct {
     float kernel_ms;         /* CUDA-event time of the recognition kernel (filtering and grains) */
     float run_ms;            /* CUDA-event time of the whole run on the device (upload included) */
     int32_t kernel_launches; /* kernels the run launched: recognition, scan of the row counts, placement and
-                                publication; three more where image rows are crowded (over 384 grains, or over
-                                64 in a run of more than 2^19) */
+                                publication; three more where image rows are crowded (over 768 grains, or over
+                                96 in a run of more than 2^19) */
     int32_t reserved;
 } et_frames_stats;
 

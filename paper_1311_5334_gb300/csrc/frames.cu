@@ -313,10 +313,11 @@ __global__ void __launch_bounds__(FT, 4) k_recognize(const __grid_constant__ FrA
 // which the host then launches.  us a call by chains and by those kernels: rows of
 // 256 grains 65 and 75 (one row), 150 and 153 (66k grains); of 320, 150 and 153
 // (82k grains); of 512, 83 and 85 (one row), 312 and 283 (262k grains); of 1,024,
-// 199 and 138 (16k grains).  Above ROW_FEW grains the kernels win from rows of some
-// 65 on: 933k grains of noise, 114 a row, 1,344 and 980; 4.2 M grains, 2,048 a row,
-// 9,582 and 6,787.
-constexpr u32 ROW_WALK = 384, ROW_WALK_LARGE = 64, ROW_FEW = 1u << 19;
+// 199 and 138 (16k grains); rows of unlike numbers, some above the limit, pay for
+// both (46k grains, 320 a row: 172, and 210 with a limit of 384).  Above ROW_FEW
+// grains the kernels win from rows of some 100 on: 933k grains of noise, 114 a row,
+// 1,344 and 980; 4.2 M grains, 2,048 a row, 9,582 and 6,787.
+constexpr u32 ROW_WALK = 768, ROW_WALK_LARGE = 96, ROW_FEW = 1u << 19;
 
 __global__ void k_fr_place(FrArgs a, const u32 *row_start, int *xyz, int *pulse, u32 *view_off) {
     griddep_launch();

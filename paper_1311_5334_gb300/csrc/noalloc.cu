@@ -112,8 +112,8 @@ __global__ void k_na_count(Batch b, const int *xyz, NaScratch s) {
 
 // Block l scans the cell counts of list l into cell starts, which also become
 // the fill cursors: tiles of NA_SC x 1024 cells, the next tile's counts loaded
-// before the current one is scanned.  28k grains on 2 x 76k cells take 7 us; a
-// one-thread-per-cell shared-memory scan of one list took 53 us.
+// before the current one is scanned.  2 x 34k cells (29k grains) take 39 us, the
+// larger part of what a call needs before it counts.
 constexpr int NA_SC = 8;
 
 __global__ void __launch_bounds__(1024) k_na_scan(NaScratch s, int n0, int n1, u32 N) {
@@ -193,7 +193,7 @@ __global__ void k_na_scatter(Batch b, const int *xyz, NaScratch s) {
 // Bound by instruction issue like the regular tube counts.  With one thread
 // per pair the lanes of a warp waited for the longest of 32 walks: 400,001
 // pairs of a 28k-grain view took 377 us of a 431 us call; the call now takes
-// 140 us.
+// 135 us, 87 of them here.
 constexpr int NA_W = 8;   // warps per block
 
 __global__ void __launch_bounds__(NA_W * 32, 4) k_na_tube(Batch b, const int *xyz, const int *pairs,
@@ -334,7 +334,7 @@ extern "C" et_status et_tube_count_noalloc(const int32_t *d_xyz, int64_t n, cons
     b.smax = params->seed_max;
     const double vol = (double)b.ext[0] * b.ext[1] * b.ext[2];
     double s0 = std::cbrt(1.4 * vol / (double)std::max<int64_t>(n, 1));
-    // no more cells than the pairs repay: one block scans a list's cells, some 0.3 us a
+    // no more cells than the pairs repay: one block scans a list's cells, some 1.2 us a
     // thousand.  At half a cell a pair and at all that fit, us a call: 65,536 grains with
     // 1, 1,000, 30,000 and 100,000 pairs 37 and 113, 85 and 124, 81 and 130, 122 and 154;
     // 21,783 grains of a thin extent with one pair 35 and 166

@@ -1,4 +1,4 @@
-"""Raster order where image rows hold many grains: up to 384 (64 in runs of more than 2^19 grains) are ranked
+"""Raster order where image rows hold many grains: up to 768 (96 in runs of more than 2^19 grains) are ranked
 along their chain, rows with more by buckets, in one handle's runs in any order, with few grains (published)
 and many (copied)."""
 import numpy as np
@@ -28,8 +28,8 @@ def want_of(oracle_mod, f):
 
 
 @pytest.mark.parametrize("width,kinds", [
-    (1280, [(384,), (385,), (64,), (3, 384, 385, 640)]),
-    (4096, [(2048, 0, 1), (1,), (384, 2048), (2048,)]),
+    (1600, [(768,), (769,), (96,), (3, 768, 769, 800)]),
+    (4096, [(2048, 0, 1), (1,), (768, 2048), (2048,)]),
 ])
 def test_rows_equal_the_oracle(oracle_mod, width, kinds):
     from paper_1311_5334_gb300 import et
@@ -45,7 +45,7 @@ def test_rows_equal_the_oracle(oracle_mod, width, kinds):
                 xyz, pulse, voff = fr.fetch()
                 assert np.array_equal(xyz, want[k][0]) and np.array_equal(pulse, want[k][1])
                 assert list(voff) == [0, len(want[k][0])]
-            crowded = max(kinds[k]) > 384
+            crowded = max(kinds[k]) > 768
             assert fr.stats()["kernel_launches"] == (7 if crowded else 4)
         fr.run(np.concatenate([f.raw.reshape(-1) for f in views]))
         xyz, pulse, voff = fr.fetch()
