@@ -92,8 +92,8 @@ def measured_peaks():
         return {}
 # DRAM bytes of the front end's recognition kernel per view of raw frames
 # (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of 8 views:
-# 441.1 MB + 7.3 MB); a launch's traffic is scaled by its view count.
-FRAMES_DRAM_BYTES_PER_VIEW = (441.1e6 + 7.3e6) / 8
+# 440.6 MB + 7.5 MB); a launch's traffic is scaled by its view count.
+FRAMES_DRAM_BYTES_PER_VIEW = (440.6e6 + 7.5e6) / 8
 
 
 def dist_env():
